@@ -18,8 +18,8 @@
  *
  * Grids: contiguous, x fastest, element (x, y, z) at x + nx*(y + ny*z);
  * 2D grids pass nz = 1.  Storage is FP32, BF16 or FP16; arithmetic is always
- * FP32 in registers and 16-bit storage is rounded (to nearest even) only
- * when a pass writes the grid back, i.e. once per `t` steps.
+ * FP32 in registers and 16-bit storage is rounded (to nearest even) once per
+ * `t` steps of the schedule (at every step by the one-step kernel).
  *
  * Conventions for every call:
  *  - Return value: STENCIL_OK (0) or a negative STENCIL_ERR_* code.  No
@@ -60,7 +60,7 @@ typedef struct stencil_plan *stencil_handle;
 typedef enum { STENCIL_F32 = 0, STENCIL_BF16 = 1, STENCIL_F16 = 2 } stencil_dtype;
 
 typedef enum {
-    STENCIL_KERNEL_AUTO = 0,   /* streaming kernel when the grid allows it, else naive */
+    STENCIL_KERNEL_AUTO = 0,   /* the library's choice (see stencil_default_schedule) */
     STENCIL_KERNEL_STREAM = 1, /* blocked streaming kernel (error if not applicable) */
     STENCIL_KERNEL_NAIVE = 2   /* one thread per cell, one step per launch (t = 1) */
 } stencil_kernel;
@@ -171,13 +171,17 @@ int stencil_run_host(stencil_handle h, const void *in_host, void *out_host, int6
                      int64_t ny, int64_t nz, int iters, int dtype, void *stream,
                      const stencil_schedule *sched);
 
-/* The schedule stencil_run would use for this problem when given none: a pick
+/* The schedule that stencil_run's results follow when it is given none: a pick
  * stored on the handle (stencil_tune with store != 0), else one stored in the
  * tuning-cache file (see stencil_tune), else the proposal of the cost model set
  * with stencil_use_cost_model, else the library's rule (2D: radius 1 at t = 4
  * with one row per step, radius 2..4 at t = 3, 2, 2 with two rows per step --
  * 16-bit storage radius 3 at t = 3 --, radius 5, 6 at t = 2; 3D: t = 2 for
- * radius 1, else t = 1; 2 rows per thread, 4 for FP32 radius 3 and 4). */
+ * radius 1, else t = 1; 2 rows per thread, 4 for FP32 radius 3 and 4; the
+ * one-step kernel for rows that are not whole 16-byte vectors).  Where it is the
+ * library's rule, 2D runs may take the same steps on register tiles instead
+ * (stencil_set_tile), with other passes and the same bits: FP32 results do not
+ * depend on the passes, and 16-bit values are rounded after the same steps. */
 int stencil_default_schedule(stencil_handle h, int64_t nx, int64_t ny, int64_t nz, int dtype,
                              stencil_schedule *out);
 
@@ -326,6 +330,15 @@ int stencil_get_device_status(void *stream, int clear);
  * never report completion, so the bounded waits of their next full pass
  * expire. */
 int stencil_set_fault_injection(stencil_handle h, int plane, int timeout_ms);
+
+/* Which kernel runs the library's rule on 2D grids: the streaming kernel or register tiles
+ * (128-cell wide tiles held in registers, any number of steps per pass; they also serve rows
+ * that are not whole 16-byte vectors).  Both give the same bits, and stencil_run,
+ * stencil_run_ex without a schedule and stencil_run_noalloc choose by estimated time; this call
+ * is for tests and measurements.  mode 0: choose (the default); -1: never tiles; 1: always tiles
+ * where they exist, with at most t steps per pass and `rows` rows per thread (0: chosen).
+ * Errors: INVALID_ARG. */
+int stencil_set_tile(stencil_handle h, int mode, int t, int rows);
 
 /* Memory-checker substitute: with on = 1, streaming sweeps on this handle use
  * the bounds-checked kernel instantiations, which test every shared-memory

@@ -31,7 +31,7 @@ KERNEL_AUTO, KERNEL_STREAM, KERNEL_NAIVE = 0, 1, 2
 # every symbol include/stencil.h declares
 EXPORTS = ("stencil_create", "stencil_create_shared", "stencil_destroy", "stencil_run", "stencil_run_ex", "stencil_run_host",
            "stencil_default_schedule", "stencil_max_t", "stencil_get_device_status",
-           "stencil_set_fault_injection", "stencil_set_checked", "stencil_run_noalloc", "stencil_run_batched", "stencil_tune",
+           "stencil_set_fault_injection", "stencil_set_checked", "stencil_set_tile", "stencil_run_noalloc", "stencil_run_batched", "stencil_tune",
            "stencil_resolve_schedule", "stencil_schedule_features", "stencil_model_create", "stencil_model_destroy",
            "stencil_model_train", "stencil_model_predict", "stencil_model_normalization",
            "stencil_model_params", "stencil_model_grad", "stencil_use_cost_model", "stencil_measure_peaks", "stencil_last_cuda_error",
@@ -101,6 +101,7 @@ def _lib():
                 lib.stencil_get_device_status.argtypes = [vp, i32]
                 lib.stencil_set_fault_injection.argtypes = [vp, i32, i32]
                 lib.stencil_set_checked.argtypes = [vp, i32]
+                lib.stencil_set_tile.argtypes = [vp, i32, i32, i32]
                 lib.stencil_run_noalloc.argtypes = [vp, vp, vp, i64, i64, i64, i32, i32, vp]
                 lib.stencil_run_batched.argtypes = [ctypes.POINTER(BatchItem), i32, vp]
                 fp = ctypes.POINTER(ctypes.c_float)
@@ -202,6 +203,11 @@ def stencil_get_device_status(stream=None, clear: bool = False) -> int:
 def stencil_set_checked(h, on: bool = True) -> int:
     """Use the bounds-checked kernel instantiations on this handle (see stencil.h)."""
     return _check(_lib().stencil_set_checked(h, 1 if on else 0), "stencil_set_checked")
+
+
+def stencil_set_tile(h, mode: int, t: int = 0, rows: int = 0) -> int:
+    """Which kernel runs the library's 2D rule (see stencil.h): 0 choose, -1 streaming, 1 register tiles."""
+    return _check(_lib().stencil_set_tile(h, mode, t, rows), "stencil_set_tile")
 
 
 def stencil_set_fault_injection(h, plane: int, timeout_ms: int = 50) -> int:

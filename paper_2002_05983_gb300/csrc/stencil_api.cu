@@ -8,6 +8,7 @@
 #include <cstdlib>
 #include <cstring>
 #include <fstream>
+#include <map>
 #include <mutex>
 #include <new>
 #include <sstream>
@@ -20,6 +21,8 @@
 #include "registry.h"
 #include "stencil.h"
 #include "sweep_kernel.cuh"
+#include "tile.h"
+#include "tile_kernel.cuh"
 
 struct stencil_plan {
     int dim = 0, r = 0, K = 0;
@@ -36,6 +39,7 @@ struct stencil_plan {
     int host_dev = -1;
     int fault_plane = -1;
     int timeout_ms = 2000;
+    int tile_mode = 0, tile_t = 0, tile_v = 0;   // test hook of the register-tile passes (stencil_set_tile)
     struct Tuned {
         int64_t nx, ny, nz;
         int dtype;
@@ -126,27 +130,34 @@ const Registry &registry()
     return reg;
 }
 
-// Functions whose shared-memory limit has been raised to the device maximum.
-std::mutex g_attr_mu;
-std::vector<const void *> g_attr_done;
+// Per function and device: registers per thread and resident blocks per SM.  The first use
+// raises the function's shared-memory limit to the device maximum; a function always launches
+// with the same block size and shared memory, so its occupancy is looked up once.
+struct FnInfo {
+    int regs = 0, occ = 0;
+};
+std::mutex g_fn_mu;
+std::map<std::pair<const void *, int>, FnInfo> g_fn;
 
-std::vector<int> g_attr_regs;   // registers per thread of each prepared function
-
-int prepare_fn(const void *fn, int max_smem, int *regs = nullptr)
+int prepare_fn(const void *fn, int threads, size_t smem, int max_smem, FnInfo *out)
 {
-    std::lock_guard<std::mutex> lk(g_attr_mu);
-    const auto it = std::find(g_attr_done.begin(), g_attr_done.end(), fn);
-    if (it != g_attr_done.end()) {
-        if (regs) *regs = g_attr_regs[static_cast<size_t>(it - g_attr_done.begin())];
+    int dev = 0;
+    CK(cudaGetDevice(&dev));
+    std::lock_guard<std::mutex> lk(g_fn_mu);
+    const auto it = g_fn.find({fn, dev});
+    if (it != g_fn.end()) {
+        *out = it->second;
         return 0;
     }
     cudaFuncAttributes fa;
     CK(cudaFuncGetAttributes(&fa, fn));   // static shared memory counts against the same limit
     CK(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize,
                             max_smem - static_cast<int>(fa.sharedSizeBytes)));
-    g_attr_done.push_back(fn);
-    g_attr_regs.push_back(fa.numRegs);
-    if (regs) *regs = fa.numRegs;
+    FnInfo f;
+    f.regs = fa.numRegs;
+    CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&f.occ, fn, threads, smem));
+    g_fn[{fn, dev}] = f;
+    *out = f;
     return 0;
 }
 
@@ -353,7 +364,8 @@ unsigned g_model_gen = 0;
 // The schedule stencil_run uses when the caller gives none: a pick stored on the handle,
 // else one in the tuning-cache file, else the active cost model's proposal, else the
 // library's rule.
-void chosen_schedule(const stencil_plan *h, int64_t nx, int64_t ny, int64_t nz, int dtype, stencil_schedule *s)
+// Returns whether it is the library's rule.
+bool chosen_schedule(const stencil_plan *h, int64_t nx, int64_t ny, int64_t nz, int dtype, stencil_schedule *s)
 {
     default_schedule(h, nx, ny, nz, dtype, s);
     bool picked = fc_lookup(h, nx, ny, nz, dtype, s);
@@ -362,7 +374,7 @@ void chosen_schedule(const stencil_plan *h, int64_t nx, int64_t ny, int64_t nz, 
             *s = tu.s;
             picked = true;
         }
-    if (picked) return;
+    if (picked) return false;
     stencil_model_handle m = nullptr;
     unsigned gen = 0;
     {
@@ -370,18 +382,19 @@ void chosen_schedule(const stencil_plan *h, int64_t nx, int64_t ny, int64_t nz, 
         m = g_model;
         gen = g_model_gen;
     }
-    if (!m || s->kernel != STENCIL_KERNEL_STREAM) return;
+    if (!m || s->kernel != STENCIL_KERNEL_STREAM) return true;
     for (const auto &mp : h->model_picks)
         if (mp.gen == gen && mp.nx == nx && mp.ny == ny && mp.nz == nz && mp.dtype == dtype) {
             *s = mp.s;
-            return;
+            return false;
         }
     stencil_schedule pick;
     if (stencil_tune(const_cast<stencil_plan *>(h), nx, ny, nz, dtype, STENCIL_TUNE_MODEL, m, 0, &pick, nullptr, 0,
                      nullptr) != STENCIL_OK)
-        return;   // keep the library's rule
+        return true;   // keep the library's rule
     *s = pick;
     h->model_picks.push_back({nx, ny, nz, dtype, gen, pick});
+    return false;
 }
 
 // Fill one pass of temporal degree t.  Pointers are set by the caller.
@@ -401,11 +414,10 @@ int plan_pass(const stencil_plan *h, int64_t nx, int64_t ny, int64_t nz, int dty
     // remainder, or fewer iterations than t) runs its own kernel's
     if (s.prefetch && t == s.t && s.prefetch != e->pf) return STENCIL_ERR_UNSUPPORTED;
     if (e->smem > static_cast<size_t>(dev.max_smem)) return STENCIL_ERR_UNSUPPORTED;
-    int regs = 0;
-    int rc = prepare_fn(e->fn, dev.max_smem, &regs);
+    FnInfo fi;
+    int rc = prepare_fn(e->fn, e->tx * e->ty, e->smem, dev.max_smem, &fi);
     if (rc) return rc;
-    int occ = 0;
-    CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, e->fn, e->tx * e->ty, e->smem));
+    const int occ = fi.occ, regs = fi.regs;
     if (occ < 1) return STENCIL_ERR_UNSUPPORTED;
 
     const int64_t ntx = (nx + e->cx - 1) / e->cx;
@@ -560,6 +572,197 @@ int launch_naive(const stencil_plan *h, const void *src, void *dst, int64_t nx, 
     return 0;
 }
 
+// ------------------------------------------------------------------------
+// Register-tile passes (tile_kernel.cuh): the other way to run the library's rule on 2D grids.
+// FP32 results do not depend on the passes, and 16-bit passes round in their registers wherever
+// the rule's own passes would end, so a run gives the same bits on either kernel.
+struct TilePlan {
+    const stn::TileEntry *e = nullptr;
+    int t = 0;              // steps per pass (the last passes may be shorter)
+    int rnd = 1;            // steps between roundings to 16-bit storage
+    double us = 0;          // estimated time of the whole run
+};
+
+const std::vector<stn::TileEntry> &tile_entries()
+{
+    static const std::vector<stn::TileEntry> all = [] {
+        std::vector<stn::TileEntry> v;
+        for (auto f : {stn::list_tile_r1, stn::list_tile_r2, stn::list_tile_r3, stn::list_tile_r4, stn::list_tile_r5,
+                       stn::list_tile_r6}) {
+            const stn::TileEntry *e = nullptr;
+            const int n = f(&e);
+            v.insert(v.end(), e, e + n);
+        }
+        return v;
+    }();
+    return all;
+}
+
+struct TileGrid {
+    int h, hx, ntx, nty;
+};
+
+// Tiles of a pass of t steps; false if the halo leaves too little of a region.
+bool tile_grid(const stn::TileEntry &e, int64_t nx, int64_t ny, int t, TileGrid *g)
+{
+    const int th = e.v * e.w;
+    g->h = e.r * t;
+    g->hx = round_up(g->h, 4);
+    if (2 * g->hx > stn::kTileW / 2 || 8 * g->h > 3 * th) return false;   // half the columns, a quarter of the rows stay
+    const int64_t cx = stn::kTileW - 2 * g->hx, cy = th - 2 * g->h;
+    const int64_t ntx = (nx + cx - 1) / cx, nty = ny <= th ? 1 : (ny - th + cy - 1) / cy + 1;
+    if (ntx * nty > 0x7fffffffLL) return false;
+    g->ntx = static_cast<int>(ntx);
+    g->nty = static_cast<int>(nty);
+    return true;
+}
+
+int tile_launch(const stencil_plan *h, const stn::TileEntry &e, int t, int rnd, const void *in, void *out, int64_t nx,
+                int64_t ny, cudaStream_t st)
+{
+    TileGrid g;
+    if (!tile_grid(e, nx, ny, t, &g)) return STENCIL_ERR_UNSUPPORTED;
+    stn::TileArgs a{};
+    a.in = in;
+    a.out = out;
+    a.nx = static_cast<int>(nx);
+    a.ny = static_cast<int>(ny);
+    a.t = t;
+    a.rnd = rnd;
+    a.h = g.h;
+    a.hx = g.hx;
+    a.ntx = g.ntx;
+    const uintptr_t vec = 4 * elem_bytes(e.dtype);   // bytes of a 4-cell vector
+    a.vin = nx % 4 == 0 && reinterpret_cast<uintptr_t>(in) % vec == 0;
+    a.vout = nx % 4 == 0 && reinterpret_cast<uintptr_t>(out) % vec == 0;
+    std::memcpy(a.c, h->c, sizeof(float) * h->K);
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3(static_cast<unsigned>(g.ntx) * static_cast<unsigned>(g.nty));
+    cfg.blockDim = dim3(static_cast<unsigned>(32 * e.w));
+    cfg.dynamicSmemBytes = e.smem;
+    cfg.stream = st;
+    // the blocks of the next pass may take their places while this one's last blocks run; they
+    // wait (griddepcontrol) for its end before they read
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    void *args[] = {&a};
+    CK(cudaLaunchKernelExC(&cfg, e.fn, args));
+    return 0;
+}
+
+// Steps of pass j of L passes over `iters` steps, as even as multiples of rnd allow.
+int tile_steps(int iters, int L, int rnd, int j)
+{
+    const int64_t units = (iters + rnd - 1) / rnd;   // the last unit may be short
+    const int64_t a = units * j / L * rnd, b = units * (j + 1) / L * rnd;
+    return static_cast<int>(std::min<int64_t>(b, iters) - a);
+}
+
+// Estimated time (us) of a pass of t steps: start + t * step + b * (block + t * block_step), b
+// tiles per SM (at least one; while they all run at once, whole tiles on the busiest SM).  The
+// constants are fits (rms 6-9 %) to measured passes over 256^2 .. 16384^2 and 256 x 16384 grids
+// at t = 1 .. 16, FP32; 16-bit storage runs within 8 % of them.  Rows per thread 4, 8 and 16.
+double tile_pass_us(const stn::TileEntry &e, const TileGrid &g, int t, int sms)
+{
+    struct Fit {
+        double start, step, block, block_step;
+    };
+    static const Fit fit[stn::kMaxR + 1][3] = {
+        {},
+        {{1.43, 0.37, 0.58, 0.104}, {1.17, 0.50, 1.08, 0.230}, {1.37, 0.80, 0.82, 0.202}},
+        {{1.29, 0.44, 0.76, 0.169}, {1.07, 0.65, 1.14, 0.361}, {1.10, 0.81, 0.95, 0.409}},
+        {{1.28, 0.50, 0.74, 0.218}, {1.14, 0.72, 1.04, 0.505}, {0.96, 0.89, 0.89, 0.527}},
+        {{1.29, 0.55, 0.74, 0.219}, {1.17, 0.90, 1.12, 0.595}, {1.28, 0.88, 0.79, 0.714}},
+        {{}, {1.31, 1.01, 0.88, 0.847}, {1.05, 1.25, 0.81, 0.925}},
+        {{}, {1.40, 1.16, 1.05, 0.913}, {1.07, 1.10, 0.98, 1.035}}};
+    const Fit &f = fit[e.r][e.v == 4 ? 0 : e.v == 8 ? 1 : 2];
+    const double n = static_cast<double>(g.ntx) * g.nty / sms;
+    const double b = n <= 1 ? 1.0 : n <= 4 ? std::ceil(n) : n + 0.3;
+    return f.start + t * f.step + b * (f.block + t * f.block_step);
+}
+
+// Estimated time (us) of the rule's streaming passes: per full pass a fixed part (launch, pipeline
+// fill, the last rows of the longest block) and a part per million cells of whole strips, fitted to
+// measured 2048^2 .. 16384^2 passes at the rule's degree.
+double stream_run_us(const stencil_plan *h, int64_t nx, int64_t ny, int dtype, int iters, const stencil_schedule &s)
+{
+    struct Fit {
+        double fixed, per_mcell;
+    };
+    static const Fit f32[stn::kMaxR + 1] = {{}, {38, 1.49}, {22, 1.59}, {22, 1.46}, {28, 1.68}, {64, 2.83}, {120, 4.30}};
+    static const Fit b16[stn::kMaxR + 1] = {{}, {43, 1.47}, {24, 1.66}, {45, 2.07}, {33, 1.74}, {66, 2.90}, {125, 4.40}};
+    // one coefficient per distance: compiled with one row per step only
+    static const double shared[stn::kMaxR + 1] = {1, 1, 1.13, 1.18, 1.26, 1, 1};
+    const Fit &f = (dtype == STENCIL_F32 ? f32 : b16)[h->r];
+    const int t = std::max(1, std::min(s.t, iters));
+    const int64_t cx = 512 - 2 * round_up((t - 1) * h->r, 4);
+    const double mcells = static_cast<double>((nx + cx - 1) / cx * cx) * static_cast<double>(ny) * 1e-6;
+    return (f.fixed + f.per_mcell * mcells) * (h->shared ? shared[h->r] : 1) * iters / s.t;
+}
+
+// Whether the rule runs this problem with register tiles, and how: the shape and the steps per
+// pass of the least estimated time, where that is below the streaming passes' (or where the rule
+// would run the one-step kernel: rows that are not whole 16-byte vectors, shared coefficients
+// without a streaming kernel).  Measured on square FP32 grids (us per step, streaming / tiles):
+// radius 1 at 256^2 12.5 / 0.7, 4096^2 15.6 / 7.7, 16384^2 109 / 98: tiles at every size; radius 2
+// 4096^2 16.5 / 14.6, 8192^2 43 / 53; radius 3 4096^2 23.2 / 20.3, 8192^2 60 / 74; radius 4 4096^2
+// 28.5 / 23.9, 8192^2 70 / 90: the line falls between; radius 6 16384^2 642 / 591.
+bool plan_tile(const stencil_plan *h, int64_t nx, int64_t ny, int dtype, int iters, const stencil_schedule &s,
+               const DevInfo &dev, TilePlan *tp)
+{
+    if (h->dim != 2 || h->checked || h->fault_plane >= 0 || h->tile_mode < 0) return false;
+    tp->rnd = s.kernel == STENCIL_KERNEL_STREAM && dtype != STENCIL_F32 ? s.t : 1;
+    tp->e = nullptr;
+    for (const auto &e : tile_entries()) {
+        if (e.r != h->r || e.dtype != dtype || e.sh != h->shared || e.smem > static_cast<size_t>(dev.max_smem)) continue;
+        if (h->tile_v && e.v != h->tile_v) continue;
+        int prev = 0;
+        for (int t = 1; t <= std::min(iters, 32); ++t) {
+            const int tu = h->tile_t ? std::min(h->tile_t, iters) : t;
+            const int unit = std::min(tp->rnd, iters);
+            if (tu % unit != 0) continue;
+            const int L = (iters + tu - 1) / tu;
+            if (L == prev) continue;   // more steps per pass, no fewer passes
+            prev = L;
+            TileGrid g;
+            const int units = (iters + unit - 1) / unit;
+            const int te = std::min((units + L - 1) / L * unit, iters);   // the longest pass
+            if (!tile_grid(e, nx, ny, te, &g)) break;
+            const double us = L * tile_pass_us(e, g, te, dev.sms);
+            if (!tp->e || us < tp->us) {
+                tp->e = &e;
+                tp->t = tu;
+                tp->us = us;
+            }
+            if (h->tile_t) break;
+        }
+    }
+    if (!tp->e) return false;
+    if (h->tile_mode > 0) return true;
+    return s.kernel != STENCIL_KERNEL_STREAM || tp->us < stream_run_us(h, nx, ny, dtype, iters, s);
+}
+
+// All passes of a run; `scratch` is the second grid of the ping-pong.
+int run_tiles(const stencil_plan *h, const TilePlan &tp, const void *in, void *out, void *scratch, int64_t nx, int64_t ny,
+              int iters, const DevInfo &dev, cudaStream_t st)
+{
+    FnInfo fi;
+    int rc = prepare_fn(tp.e->fn, 32 * tp.e->w, tp.e->smem, dev.max_smem, &fi);
+    if (rc) return rc;
+    const int L = (iters + tp.t - 1) / tp.t, unit = std::min(tp.rnd, iters);
+    const void *src = in;
+    for (int j = 0; j < L; ++j) {
+        void *dst = ((L - 1 - j) % 2 == 0) ? out : scratch;
+        rc = tile_launch(h, *tp.e, tile_steps(iters, L, unit, j), unit, src, dst, nx, ny, st);
+        if (rc) return rc;
+        src = dst;
+    }
+    return 0;
+}
+
 int run_impl(stencil_plan *h, const void *in, void *out, int64_t nx, int64_t ny, int64_t nz,
              int iters, int dtype, cudaStream_t st, const stencil_schedule *user)
 {
@@ -574,7 +777,9 @@ int run_impl(stencil_plan *h, const void *in, void *out, int64_t nx, int64_t ny,
         return 0;
     }
     stencil_schedule s;
-    chosen_schedule(h, nx, ny, nz, dtype, &s);
+    const bool rule = chosen_schedule(h, nx, ny, nz, dtype, &s);
+    static const stencil_schedule kNone{};
+    const bool plain = !user || std::memcmp(user, &kNone, sizeof(kNone)) == 0;
     if (user) {
         if (user->kernel < 0 || user->kernel > STENCIL_KERNEL_NAIVE) return STENCIL_ERR_INVALID_ARG;
         if (user->kernel) s.kernel = user->kernel;
@@ -594,6 +799,15 @@ int run_impl(stencil_plan *h, const void *in, void *out, int64_t nx, int64_t ny,
     const bool streamable = stream_applicable(dtype, nx) && aligned;
     if (s.kernel == STENCIL_KERNEL_STREAM && !streamable) return STENCIL_ERR_UNSUPPORTED;
     if (s.kernel == STENCIL_KERNEL_AUTO) s.kernel = streamable ? STENCIL_KERNEL_STREAM : STENCIL_KERNEL_NAIVE;
+
+    TilePlan tp;
+    if (rule && plain && plan_tile(h, nx, ny, dtype, iters, s, *dev, &tp)) {
+        if (iters > tp.t) {
+            rc = ensure_scratch(h, bytes);
+            if (rc) return rc;
+        }
+        return run_tiles(h, tp, in, out, h->scratch, nx, ny, iters, *dev, st);
+    }
 
     // passes: full passes of degree t, then the remainder
     std::vector<int> degrees;
@@ -927,10 +1141,10 @@ int build_batch(const stencil_batch_item *items, int n, const DevInfo &dev, cuda
             c.phase = phase;
             c.block = dim3(kind->tx, kind->ty);
             c.smem = kind->smem;
-            int rc = prepare_fn(c.pfn, dev.max_smem);
+            FnInfo fi;
+            int rc = prepare_fn(c.pfn, kind->tx * kind->ty, kind->smem, dev.max_smem, &fi);
             if (rc) return rc;
-            int occ = 0;
-            CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, c.pfn, kind->tx * kind->ty, kind->smem));
+            const int occ = fi.occ;
             if (occ < 1) return STENCIL_ERR_UNSUPPORTED;
             c.grid = dim3(static_cast<unsigned>(std::min<int64_t>(total, static_cast<int64_t>(dev.sms) * occ)));
             const int nt = static_cast<int>(tasks.size());
@@ -1192,6 +1406,15 @@ int stencil_set_checked(stencil_handle h, int on)
     return STENCIL_OK;
 }
 
+int stencil_set_tile(stencil_handle h, int mode, int t, int rows)
+{
+    if (!h || mode < -1 || mode > 1 || t < 0 || rows < 0) return STENCIL_ERR_INVALID_ARG;
+    h->tile_mode = mode;
+    h->tile_t = mode > 0 ? t : 0;
+    h->tile_v = mode > 0 ? rows : 0;
+    return STENCIL_OK;
+}
+
 int stencil_set_fault_injection(stencil_handle h, int plane, int timeout_ms)
 {
     if (!h) return STENCIL_ERR_INVALID_ARG;
@@ -1231,6 +1454,9 @@ int stencil_run_noalloc(stencil_handle h, const void *in, void *out, int64_t nx,
     default_schedule(h, nx, ny, nz, dtype, &s);
     const bool aligned = (reinterpret_cast<uintptr_t>(in) | reinterpret_cast<uintptr_t>(out)) % 16 == 0;
     const bool streamable = s.kernel == STENCIL_KERNEL_STREAM && aligned;
+    TilePlan tp;
+    if (aligned && plan_tile(h, nx, ny, dtype, iters, s, dev, &tp))
+        return run_tiles(h, tp, in, out, nd->scratch, nx, ny, iters, dev, st);
     const int t = streamable ? std::max(1, std::min(s.t, iters)) : 1;
     const int L = (iters + t - 1) / t;
     const int t_last = iters - (L - 1) * t;
