@@ -173,6 +173,16 @@ __device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c)
     return d;
 }
 
+// Programmatic dependent launch (a pass launched as a programmatic dependent of the pass before
+// it): the next pass's blocks may take their places as soon as every block of this one has
+// started, and set themselves up; they read and write grids only after grid_dep_wait, which
+// returns when all work before this launch is complete (at once in any other launch).  3D passes
+// use it (512^3, radius 1..4: 1 % faster; 96^3, one-wave blocks: 6.8 -> 5.9 us per pass); 2D
+// streaming passes don't: blocks placed as slots come free lose the order in which neighbouring
+// strips share L2 (16384^2 radius 4 0.4 %, 8192^2 2.6 % slower with it).
+__device__ __forceinline__ void grid_dep_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void grid_dep_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
 // --------------------------------------------------------- storage formats
 template <typename S> struct Fmt;
 template <> struct Fmt<float> {
@@ -704,6 +714,7 @@ __device__ __forceinline__ bool sweep_tile(const CUtensorMap *tmap, const SweepA
             tma_load_3d(smem_addr(dst0), tmap, ox_in, oy, q, bar);
         }
     };
+    if constexpr (D == 3) grid_dep_wait();   // the set-up above overlaps the end of the pass before
     {
         const int qe = min(k0 + G::PFS - 1, smax);
         if (tid == 0)
@@ -1186,6 +1197,7 @@ __global__ void __launch_bounds__(TX *TY)
     sweep_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_constant__ SweepArgs a)
 {
     extern __shared__ __align__(1024) unsigned char smem[];
+    if constexpr (D == 3) grid_dep_launch();
     sweep_block<D, R, T, VY, S, TX, TY, SH, CHK, P>(&tmap, a, static_cast<int>(blockIdx.x), smem);
 }
 

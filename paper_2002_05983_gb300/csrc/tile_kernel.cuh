@@ -279,9 +279,6 @@ __device__ __forceinline__ void tile2d(const A &a, int blk, float4 *halo)
     }
 }
 
-__device__ __forceinline__ void grid_dep_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
-__device__ __forceinline__ void grid_dep_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
-
 // One pass over the grid, one tile per block.
 template <int R, int V, int W, typename S, bool SH>
 __global__ void __launch_bounds__(32 * W, V <= 8 ? 2 : 1) tile2d_kernel(const __grid_constant__ TileArgs a)
