@@ -290,22 +290,22 @@ typedef struct {
 
 /* Sweep many independent grids of mixed dimension, radius and storage type
  * together (not in the paper; a serving-style batch of the paper's sweep).
- * Each grid runs exactly the passes stencil_run would: iters / t passes of its
- * handle's tuned or default degree t, then one remainder pass of degree
- * iters mod t, so results equal stencil_run's bit for bit.  Passes are grouped
- * by kernel class (dim, radius, dtype, temporal degree, rows per thread or per
- * step); each class runs as ONE persistent launch whose blocks take tiles from
- * a device-side queue ordered pass by pass over all grids of the class,
- * largest grids first; a tile of pass p of a grid starts only when all tiles
- * of its pass p-1 are done (bounded wait: on expiry the device status is set,
- * see stencil_get_device_status).  All class launches of the full passes are
- * captured as parallel branches of one CUDA graph, so the classes run side by
- * side and one class's last wave overlaps the others' work; the remainder
- * passes follow as a second set of parallel branches once every full pass is
- * done.  The graph is cached for this exact item list (same pointers, sizes,
- * handles, schedules) and replayed on `stream` by later calls.  The batch owns
- * one scratch grid per item (allocated on the first call for an item list,
- * before capture) and keeps up to four cached lists.
+ * Results equal stencil_run's bit for bit.  The list becomes one CUDA graph that
+ * is cached for this exact item list (same pointers, sizes, handles, schedules)
+ * and replayed on `stream` by later calls: every grid is a chain of the passes
+ * stencil_run would launch; the 2D grids, whose passes fill the device, follow
+ * one another, and each 3D grid runs on a parallel branch in passes cut for its
+ * part of the device.  Lists of more than 20000 passes, whose graphs would grow
+ * too large, and handles with the fault-injection or checked hooks run as
+ * persistent launches instead, one per kernel class (dim, radius, dtype,
+ * temporal degree, rows per thread or per step) on parallel graph branches:
+ * iters / t passes of each grid's tuned or default degree t, then one remainder
+ * pass, blocks taking tiles from a device-side queue ordered pass by pass over
+ * all grids of the class, largest grids first; a tile of pass p of a grid starts
+ * only when all tiles of its pass p-1 are done (bounded wait: on expiry the
+ * device status is set, see stencil_get_device_status).  The batch owns one
+ * allocation for the scratch grids of its items (made on the first call for an
+ * item list, before capture) and keeps up to four cached lists.
  * Every grid must allow the streaming kernel (rows 16-byte aligned: nx % 4
  * FP32, nx % 8 16-bit; 16-byte aligned pointers), else STENCIL_ERR_UNSUPPORTED.
  * Items may share a handle; `in` of one item must not overlap any `out`.

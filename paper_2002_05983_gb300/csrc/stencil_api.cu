@@ -422,8 +422,10 @@ int64_t whole_wave_seg(int64_t tiles, int64_t ns, int64_t slots, int64_t halo)
 }
 
 // Fill one pass of temporal degree t.  Pointers are set by the caller.
+// batched: tiles of a persistent launch.  share: the part of the device this pass is meant to fill
+// (1: it has the device to itself).
 int plan_pass(const stencil_plan *h, int64_t nx, int64_t ny, int64_t nz, int dtype, int t,
-              const stencil_schedule &s, const DevInfo &dev, Pass &ps, bool batched = false)
+              const stencil_schedule &s, const DevInfo &dev, Pass &ps, bool batched = false, double share = 1.0)
 {
     const int D = h->dim, R = h->r;
     const int vy = D == 3 ? s.rows_per_thread : 1;
@@ -467,7 +469,8 @@ int plan_pass(const stencil_plan *h, int64_t nx, int64_t ny, int64_t nz, int dty
             // >= 4 waves (dynamic balance of edge tiles), segments long against the fill
             const int64_t want = (4 * slots + tiles - 1) / tiles;
             seg = std::max<int64_t>((ns + want - 1) / want, minseg);
-            if (D == 3 && !batched && tiles * ((ns + seg - 1) / seg) < 3 * slots) seg = whole_wave_seg(tiles, ns, slots, 2 * R * t);
+            if (D == 3 && !batched && (share < 1 || tiles * ((ns + seg - 1) / seg) < 3 * slots))
+                seg = whole_wave_seg(tiles, ns, std::max<int64_t>(1, static_cast<int64_t>(static_cast<double>(slots) * share)), 2 * R * t);
         } else if (batched) {
             // other grids fill the device: segments long against the pipeline fill
             seg = std::max<int64_t>((W + 4 * slots - 1) / (4 * slots), minseg);
@@ -795,6 +798,40 @@ int run_tiles(const stencil_plan *h, const TilePlan &tp, const void *in, void *o
     return 0;
 }
 
+// All streaming passes of a run: full passes of the schedule's degree, then the remainder.
+// `scratch` is the second grid of the ping-pong.
+int run_stream(const stencil_plan *h, const void *in, void *out, void *scratch, int64_t nx, int64_t ny, int64_t nz, int iters,
+               int dtype, const stencil_schedule &s, const DevInfo &dev, cudaStream_t st, double share = 1.0)
+{
+    const int t = std::max(1, std::min(s.t, iters)), L = (iters + t - 1) / t, t_last = iters - (L - 1) * t;
+    Pass full, tail;
+    int rc = plan_pass(h, nx, ny, nz, dtype, t, s, dev, full, false, share);
+    if (rc) return rc;
+    if (t_last != t) {
+        rc = plan_pass(h, nx, ny, nz, dtype, t_last, s, dev, tail, false, share);
+        if (rc) return rc;
+    }
+    const void *src = in;
+    for (int j = 0; j < L; ++j) {
+        void *dst = ((L - 1 - j) % 2 == 0) ? out : scratch;
+        Pass &ps = (j == L - 1 && t_last != t) ? tail : full;
+        ps.a.in = src;
+        ps.a.out = dst;
+        CUtensorMap map;
+        std::memset(&map, 0, sizeof(map));
+        if (h->dim == 3) {
+            rc = encode_map(&map, src, nx, ny, nz, dtype, 4 * static_cast<int>(ps.block.x) + 2 * ps.padin,
+                            static_cast<int>(ps.block.y) * s.rows_per_thread + 2 * h->r);
+            if (rc) return rc;
+        }
+        void *args[] = {&map, &ps.a};
+        rc = launch_pass(ps.fn, ps.grid, ps.block, args, ps.smem, st, h->dim == 3);
+        if (rc) return rc;
+        src = dst;
+    }
+    return 0;
+}
+
 int run_impl(stencil_plan *h, const void *in, void *out, int64_t nx, int64_t ny, int64_t nz,
              int iters, int dtype, cudaStream_t st, const stencil_schedule *user)
 {
@@ -841,49 +878,17 @@ int run_impl(stencil_plan *h, const void *in, void *out, int64_t nx, int64_t ny,
         return run_tiles(h, tp, in, out, h->scratch, nx, ny, iters, *dev, st);
     }
 
-    // passes: full passes of degree t, then the remainder
-    std::vector<int> degrees;
     const int t = s.kernel == STENCIL_KERNEL_NAIVE ? 1 : std::max(1, std::min(s.t, iters));
-    for (int done = 0; done < iters; done += t) degrees.push_back(std::min(t, iters - done));
-    const int L = static_cast<int>(degrees.size());
-    if (L > 1) {
+    if (iters > t) {
         rc = ensure_scratch(h, bytes);
         if (rc) return rc;
     }
-    std::vector<Pass> plans;
-    if (s.kernel == STENCIL_KERNEL_STREAM) {
-        for (int j = 0; j < L; ++j) {
-            if (j > 0 && degrees[j] == degrees[j - 1]) {
-                plans.push_back(plans.back());
-                continue;
-            }
-            Pass ps;
-            rc = plan_pass(h, nx, ny, nz, dtype, degrees[j], s, *dev, ps);
-            if (rc) return rc;
-            plans.push_back(ps);
-        }
-    }
+    if (s.kernel == STENCIL_KERNEL_STREAM) return run_stream(h, in, out, h->scratch, nx, ny, nz, iters, dtype, s, *dev, st);
     const void *src = in;
-    for (int j = 0; j < L; ++j) {
-        void *dst = ((L - 1 - j) % 2 == 0) ? out : h->scratch;
-        if (s.kernel == STENCIL_KERNEL_NAIVE) {
-            rc = launch_naive(h, src, dst, nx, ny, nz, dtype, st, *dev);
-            if (rc) return rc;
-        } else {
-            Pass &ps = plans[j];
-            ps.a.in = src;
-            ps.a.out = dst;
-            CUtensorMap map;
-            std::memset(&map, 0, sizeof(map));
-            if (h->dim == 3) {
-                rc = encode_map(&map, src, nx, ny, nz, dtype, 4 * static_cast<int>(ps.block.x) + 2 * ps.padin,
-                                static_cast<int>(ps.block.y) * s.rows_per_thread + 2 * h->r);
-                if (rc) return rc;
-            }
-            void *args[] = {&map, &ps.a};
-            rc = launch_pass(ps.fn, ps.grid, ps.block, args, ps.smem, st, h->dim == 3);
-            if (rc) return rc;
-        }
+    for (int j = 0; j < iters; ++j) {
+        void *dst = ((iters - 1 - j) % 2 == 0) ? out : h->scratch;
+        rc = launch_naive(h, src, dst, nx, ny, nz, dtype, st, *dev);
+        if (rc) return rc;
         src = dst;
     }
     return 0;
@@ -1024,7 +1029,8 @@ int candidates(const stencil_plan *h, int64_t ny, int64_t nz, int dtype, stencil
 }
 
 // ------------------------------------------------------------------------
-// Batched persistent sweeps: plans, device task tables and cached CUDA graphs.
+// Batched sweeps: plans, the graph of chains or the persistent launches with their device task
+// tables, and the cache of both.
 struct BatchClass {
     const void *pfn = nullptr;
     int phase = 0;                 // 0: full passes of every grid; 1: remainder passes
@@ -1036,6 +1042,7 @@ struct BatchClass {
 
 struct BatchEntry {
     std::vector<char> key;
+    void *scratch_mem = nullptr;   // one allocation for the scratch grids of all items
     std::vector<void *> scratch;   // one per item (null when a grid needs a single pass)
     std::vector<BatchClass> classes;
     cudaGraphExec_t exec = nullptr;
@@ -1049,8 +1056,7 @@ void free_entry(BatchEntry *e)
 {
     cudaDeviceSynchronize();   // a replay may still use the tables
     if (e->exec) cudaGraphExecDestroy(e->exec);
-    for (void *p : e->scratch)
-        if (p) cudaFree(p);
+    if (e->scratch_mem) cudaFree(e->scratch_mem);
     for (auto &c : e->classes) {
         for (void *p : {c.dev_args, c.dev_maps, c.dev_tasks, c.dev_done})
             if (p) cudaFree(p);
@@ -1067,18 +1073,163 @@ std::vector<char> batch_key(const stencil_batch_item *items, int n, int dev)
         const stencil_plan *h = items[i].h;
         const char *c = reinterpret_cast<const char *>(h->c);
         k.insert(k.end(), c, c + sizeof(float) * h->K);
-        int extra[3] = {h->fault_plane, h->timeout_ms, h->kind()};   // kind: shared / checked kernels
+        int extra[6] = {h->fault_plane, h->timeout_ms, h->kind(), h->tile_mode, h->tile_t, h->tile_v};   // kind: shared / checked kernels
         k.insert(k.end(), reinterpret_cast<char *>(extra), reinterpret_cast<char *>(extra) + sizeof(extra));
         stencil_schedule sc;   // the schedule the batch will use for this grid
-        chosen_schedule(h, items[i].nx, items[i].ny, items[i].nz, items[i].dtype, &sc);
+        k.push_back(chosen_schedule(h, items[i].nx, items[i].ny, items[i].nz, items[i].dtype, &sc) ? 1 : 0);
         const char *b = reinterpret_cast<const char *>(&sc);
         k.insert(k.end(), b, b + sizeof(sc));
     }
     return k;
 }
 
+// Scratch grids (the second buffer of each grid's ping-pong) in one allocation.
+int batch_scratch(const stencil_batch_item *items, int n, const std::vector<int> &npass, BatchEntry *E)
+{
+    E->scratch.assign(n, nullptr);
+    std::vector<size_t> at(n, 0);
+    size_t total = 0;
+    for (int i = 0; i < n; ++i)
+        if (npass[i] > 1) {
+            at[i] = total;
+            total += (static_cast<size_t>(items[i].nx * items[i].ny * items[i].nz) * elem_bytes(items[i].dtype) + 255) / 256 * 256;
+        }
+    if (!total) return 0;
+    CK(cudaMalloc(&E->scratch_mem, total));
+    for (int i = 0; i < n; ++i)
+        if (npass[i] > 1) E->scratch[i] = static_cast<char *>(E->scratch_mem) + at[i];
+    return 0;
+}
+
+// One grid of a batch as a chain of the passes stencil_run would launch.
+struct BatchChain {
+    int item = 0;
+    bool tiles = false;
+    TilePlan tp;
+    stencil_schedule s{};
+    double us = 0;        // estimated time with the device to itself
+    int passes = 0;
+    int branch = 0;
+};
+
+// Chains of at most this many launches in all become a graph of ordinary passes; longer lists (and
+// handles with test hooks) keep the persistent launches, whose size does not grow with the steps.
+constexpr int64_t kMaxChainNodes = 20000;
+
+// Plans every grid's chain; returns false (rc = 0) where the list runs as persistent launches.
+bool plan_chains(const stencil_batch_item *items, int n, const DevInfo &dev, std::vector<BatchChain> *out, int *rc)
+{
+    *rc = 0;
+    int64_t nodes = 0;
+    for (int i = 0; i < n; ++i) {
+        const stencil_batch_item &b = items[i];
+        BatchChain c;
+        c.item = i;
+        const bool rule = chosen_schedule(b.h, b.nx, b.ny, b.nz, b.dtype, &c.s);
+        if (c.s.kernel != STENCIL_KERNEL_STREAM) {
+            *rc = STENCIL_ERR_UNSUPPORTED;
+            return false;
+        }
+        if (b.h->checked || b.h->fault_plane >= 0) return false;
+        c.tiles = rule && plan_tile(b.h, b.nx, b.ny, b.dtype, b.iters, c.s, dev, &c.tp);
+        // microseconds per million cell updates of the streaming kernels at the rule's degrees
+        static const double us3[stn::kMaxR + 1] = {0, 0.87, 1.25, 1.35, 1.6, 2.5, 3.2};
+        c.us = c.tiles ? c.tp.us
+               : b.h->dim == 2 ? stream_run_us(b.h, b.nx, b.ny, b.dtype, b.iters, c.s)
+                               : us3[b.h->r] * 1e-6 * static_cast<double>(b.nx * b.ny * b.nz) * b.iters;
+        const int t = c.tiles ? c.tp.t : std::max(1, std::min(c.s.t, b.iters));
+        c.passes = (b.iters + t - 1) / t;
+        nodes += c.passes;
+        out->push_back(c);
+    }
+    return nodes <= kMaxChainNodes;
+}
+
+// One CUDA graph of the grids' chains.  2D passes fill the device, so the 2D grids follow one another
+// on one branch.  A 3D pass of a small grid does not, and cutting it into enough blocks to do so
+// spends most of the planes on halos; every 3D grid has a branch of its own, at high priority, whose
+// passes are cut for six times its share of the batch's work, so the 3D chains run beside the 2D
+// one.  Measured on 16 2D + 8 3D grids, 100 steps: 62 ms as persistent launches per kernel class
+// (a class's blocks hold the SMs until it ends, so a grid of a few tiles runs nearly alone), 46 ms as
+// one chain, 43.5 ms so; cutting for 1.5 / 3 / 12 times the share 54 / 47 / 45 ms, two 2D branches
+// 45 ms; 5 + 3 grids 12.3 -> 7.7 ms, 12 + 2 37.2 -> 21.4, 2 + 8 10.4 -> 5.9.
+int build_chains(const stencil_batch_item *items, std::vector<BatchChain> &chains, const DevInfo &dev, BatchEntry *E)
+{
+    const int n = static_cast<int>(chains.size());
+    std::vector<int> npass(n);
+    double total = 0;
+    for (const auto &c : chains) {
+        npass[c.item] = c.passes;
+        total += c.us;
+    }
+    int rc = batch_scratch(items, n, npass, E);
+    if (rc) return rc;
+    std::vector<BatchChain *> order;
+    for (auto &c : chains) order.push_back(&c);
+    std::stable_sort(order.begin(), order.end(), [](const BatchChain *a, const BatchChain *b) { return a->us > b->us; });
+    constexpr int k2 = 1, k3 = 16;   // branches of 2D grids; at most so many of 3D grids
+    double load[k2 + k3] = {};
+    int n3 = 0;
+    for (auto *c : order) {   // longest first onto the least loaded branch of its kind
+        const bool two = items[c->item].h->dim == 2;
+        int best = two ? 0 : k2;
+        for (int k = best; k < (two ? k2 : k2 + k3); ++k)
+            if (load[k] < load[best]) best = k;
+        c->branch = best;
+        load[best] += c->us;
+        if (!two) n3 = std::max(n3, best - k2 + 1);
+    }
+    const int nb = k2 + n3;
+    int lo = 0, hi = 0;
+    CK(cudaDeviceGetStreamPriorityRange(&lo, &hi));
+    std::vector<cudaStream_t> br(nb, nullptr);
+    std::vector<cudaEvent_t> ev(nb + 1, nullptr);
+    cudaStream_t cap = nullptr;
+    cudaError_t err = cudaStreamCreateWithFlags(&cap, cudaStreamNonBlocking);
+    for (int k = 0; k < nb; ++k)
+        if (err == cudaSuccess) err = cudaStreamCreateWithPriority(&br[k], cudaStreamNonBlocking, k < k2 ? lo : hi);
+    for (auto &x : ev)
+        if (err == cudaSuccess) err = cudaEventCreateWithFlags(&x, cudaEventDisableTiming);
+    cudaGraph_t graph = nullptr;
+    if (err == cudaSuccess) err = cudaStreamBeginCapture(cap, cudaStreamCaptureModeThreadLocal);
+    if (err == cudaSuccess) {
+        err = cudaEventRecord(ev[nb], cap);
+        for (int k = 0; k < nb && err == cudaSuccess; ++k) err = cudaStreamWaitEvent(br[k], ev[nb], 0);
+        for (auto *c : order) {
+            if (rc || err != cudaSuccess) break;
+            const stencil_batch_item &b = items[c->item];
+            void *scr = E->scratch[c->item];
+            if (c->tiles)
+                rc = run_tiles(b.h, c->tp, b.in, b.out, scr, b.nx, b.ny, b.iters, dev, br[c->branch]);
+            else
+                rc = run_stream(b.h, b.in, b.out, scr, b.nx, b.ny, b.nz, b.iters, b.dtype, c->s, dev, br[c->branch],
+                                b.h->dim == 3 ? std::min(1.0, 6.0 * c->us / total) : 1.0);
+        }
+        for (int k = 0; k < nb && err == cudaSuccess; ++k) {
+            err = cudaEventRecord(ev[k], br[k]);
+            if (err == cudaSuccess) err = cudaStreamWaitEvent(cap, ev[k], 0);
+        }
+        const cudaError_t e2 = cudaStreamEndCapture(cap, &graph);
+        if (err == cudaSuccess) err = e2;
+    }
+    if (!rc && err == cudaSuccess) err = cudaGraphInstantiate(&E->exec, graph, 0);
+    if (graph) cudaGraphDestroy(graph);
+    for (auto x : ev)
+        if (x) cudaEventDestroy(x);
+    for (auto x : br)
+        if (x) cudaStreamDestroy(x);
+    if (cap) cudaStreamDestroy(cap);
+    if (rc) return rc;
+    if (err != cudaSuccess) return cuda_fail(err, __LINE__);
+    return 0;
+}
+
 int build_batch(const stencil_batch_item *items, int n, const DevInfo &dev, cudaStream_t st, BatchEntry *E)
 {
+    std::vector<BatchChain> chains;
+    int crc = 0;
+    if (plan_chains(items, n, dev, &chains, &crc)) return build_chains(items, chains, dev, E);
+    if (crc) return crc;
     // Every grid runs ceil(iters / t) passes at its own chosen degree t, like stencil_run:
     // L = iters / t full passes (phase 0), then one remainder pass of degree iters mod t
     // (phase 1).  Each pass becomes a task of the kernel class that sweeps it.
@@ -1112,14 +1263,8 @@ int build_batch(const stencil_batch_item *items, int n, const DevInfo &dev, cuda
             passes.push_back(x);
         }
     }
-    // scratch grids (the second buffer of each grid's ping-pong)
-    E->scratch.assign(n, nullptr);
-    for (int i = 0; i < n; ++i)
-        if (npass[i] > 1) {
-            const stencil_batch_item &b = items[i];
-            const size_t bytes = static_cast<size_t>(b.nx * b.ny * b.nz) * elem_bytes(b.dtype);
-            CK(cudaMalloc(&E->scratch[i], bytes));
-        }
+    int rcs = batch_scratch(items, n, npass, E);
+    if (rcs) return rcs;
     // kernel classes per phase; inside a class, tasks pass-major, largest grids first, so every
     // tile a block waits for was taken earlier by a running block of the same class
     for (int phase = 0; phase < 2; ++phase) {
@@ -1490,40 +1635,12 @@ int stencil_run_noalloc(stencil_handle h, const void *in, void *out, int64_t nx,
     TilePlan tp;
     if (aligned && plan_tile(h, nx, ny, dtype, iters, s, dev, &tp))
         return run_tiles(h, tp, in, out, nd->scratch, nx, ny, iters, dev, st);
-    const int t = streamable ? std::max(1, std::min(s.t, iters)) : 1;
-    const int L = (iters + t - 1) / t;
-    const int t_last = iters - (L - 1) * t;
-    Pass full, tail;
-    if (streamable) {
-        rc = plan_pass(h, nx, ny, nz, dtype, t, s, dev, full);
-        if (rc) return rc;
-        if (t_last != t) {
-            rc = plan_pass(h, nx, ny, nz, dtype, t_last, s, dev, tail);
-            if (rc) return rc;
-        }
-    }
+    if (streamable) return run_stream(h, in, out, nd->scratch, nx, ny, nz, iters, dtype, s, dev, st);
     const void *src = in;
-    for (int j = 0; j < L; ++j) {
-        void *dst = ((L - 1 - j) % 2 == 0) ? out : nd->scratch;
-        if (!streamable) {
-            rc = launch_naive(h, src, dst, nx, ny, nz, dtype, st, dev);
-            if (rc) return rc;
-        } else {
-            Pass &ps = (j == L - 1 && t_last != t) ? tail : full;
-            ps.a.in = src;
-            ps.a.out = dst;
-            ps.a.status = nd->status;
-            CUtensorMap map;
-            std::memset(&map, 0, sizeof(map));
-            if (h->dim == 3) {
-                rc = encode_map(&map, src, nx, ny, nz, dtype, 4 * static_cast<int>(ps.block.x) + 2 * ps.padin,
-                                static_cast<int>(ps.block.y) * s.rows_per_thread + 2 * h->r);
-                if (rc) return rc;
-            }
-            void *args[] = {&map, &ps.a};
-            rc = launch_pass(ps.fn, ps.grid, ps.block, args, ps.smem, st, h->dim == 3);
-            if (rc) return rc;
-        }
+    for (int j = 0; j < iters; ++j) {
+        void *dst = ((iters - 1 - j) % 2 == 0) ? out : nd->scratch;
+        rc = launch_naive(h, src, dst, nx, ny, nz, dtype, st, dev);
+        if (rc) return rc;
         src = dst;
     }
     return STENCIL_OK;
