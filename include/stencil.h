@@ -179,7 +179,7 @@ int stencil_run_host(stencil_handle h, const void *in_host, void *out_host, int6
  * 16-bit storage radius 3 at t = 3 --, radius 5, 6 at t = 2; 3D: t = 2 for
  * radius 1, else t = 1; 2 rows per thread, 4 for FP32 radius 3 and 4; the
  * one-step kernel for rows that are not whole 16-byte vectors).  Where it is the
- * library's rule, 2D runs may take the same steps on register tiles instead
+ * library's rule, runs may take the same steps on other kernels
  * (stencil_set_tile), with other passes and the same bits: FP32 results do not
  * depend on the passes, and 16-bit values are rounded after the same steps. */
 int stencil_default_schedule(stencil_handle h, int64_t nx, int64_t ny, int64_t nz, int dtype,
@@ -331,12 +331,13 @@ int stencil_get_device_status(void *stream, int clear);
  * expire. */
 int stencil_set_fault_injection(stencil_handle h, int plane, int timeout_ms);
 
-/* Which kernel runs the library's rule on 2D grids: the streaming kernel or register tiles
- * (128-cell wide tiles held in registers, any number of steps per pass; they also serve rows
- * that are not whole 16-byte vectors).  Both give the same bits, and stencil_run,
- * stencil_run_ex without a schedule and stencil_run_noalloc choose by estimated time; this call
- * is for tests and measurements.  mode 0: choose (the default); -1: never tiles; 1: always tiles
- * where they exist, with at most t steps per pass and `rows` rows per thread (0: chosen).
+/* Which kernels run the library's rule.  2D grids run streaming passes or register tiles (128-cell
+ * wide tiles held in registers, any number of steps per pass, rows of any length); 3D grids whose
+ * rows are not whole 16-byte vectors run the one-step kernel or, on a padded copy, streaming passes
+ * for rows of any length.  All give the same bits, and stencil_run, stencil_run_ex without a
+ * schedule and stencil_run_noalloc choose by estimated time; this call is for tests and
+ * measurements.  mode 0: choose (the default); -1: never tiles nor padded copies; 1: always where
+ * they exist, tiles with at most t steps per pass and `rows` rows per thread (0: chosen).
  * Errors: INVALID_ARG. */
 int stencil_set_tile(stencil_handle h, int mode, int t, int rows);
 

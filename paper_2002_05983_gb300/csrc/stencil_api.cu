@@ -18,6 +18,7 @@
 #include <cudaTypedefs.h>
 
 #include "naive.h"
+#include "pack.h"
 #include "registry.h"
 #include "stencil.h"
 #include "sweep_kernel.cuh"
@@ -97,7 +98,9 @@ struct Registry {
                            stn::list_3d_bf16_r5, stn::list_3d_bf16_r6, stn::list_2d_f16_r5,
                            stn::list_2d_f16_r6,  stn::list_3d_f16_r5,  stn::list_3d_f16_r6,
                            stn::list_2d_f32sh,   stn::list_3d_f32sh,   stn::list_checked,  stn::list_2d_f32_p2,
-                           stn::list_2d_bf16_p2, stn::list_2d_f16_p2,  stn::list_2d_p4};
+                           stn::list_2d_bf16_p2, stn::list_2d_f16_p2,  stn::list_2d_p4,
+                           stn::list_rag_f32,    stn::list_rag_f32_wide, stn::list_rag_bf16,  stn::list_rag_f16,
+                           stn::list_rag_2d};
         for (L f : lists) {
             const stn::KernelEntry *e = nullptr;
             const int n = f(&e);
@@ -423,17 +426,18 @@ int64_t whole_wave_seg(int64_t tiles, int64_t ns, int64_t slots, int64_t halo)
 
 // Fill one pass of temporal degree t.  Pointers are set by the caller.
 // batched: tiles of a persistent launch.  share: the part of the device this pass is meant to fill
-// (1: it has the device to itself).
+// (1: it has the device to itself).  kind: the registry's kernel variant (default the handle's).
 int plan_pass(const stencil_plan *h, int64_t nx, int64_t ny, int64_t nz, int dtype, int t,
-              const stencil_schedule &s, const DevInfo &dev, Pass &ps, bool batched = false, double share = 1.0)
+              const stencil_schedule &s, const DevInfo &dev, Pass &ps, bool batched = false, double share = 1.0, int kind = -1)
 {
+    if (kind < 0) kind = h->kind();
     const int D = h->dim, R = h->r;
     const int vy = D == 3 ? s.rows_per_thread : 1;
     int pps = D == 2 && s.planes_per_step ? s.planes_per_step : 1;
-    const stn::KernelEntry *e = registry().find(D, R, t, vy, dtype, h->kind(), s.threads_x, D == 3 ? s.threads_y : 0, pps);
+    const stn::KernelEntry *e = registry().find(D, R, t, vy, dtype, kind, s.threads_x, D == 3 ? s.threads_y : 0, pps);
     while (!e && pps > 1) {   // a degree compiled with fewer rows per step (e.g. a remainder pass)
         pps /= 2;
-        e = registry().find(D, R, t, vy, dtype, h->kind(), s.threads_x, 0, pps);
+        e = registry().find(D, R, t, vy, dtype, kind, s.threads_x, 0, pps);
     }
     if (!e) return STENCIL_ERR_UNSUPPORTED;
     // the prefetch depth is a property of the degree-t kernel; a pass of another degree (the
@@ -512,14 +516,15 @@ int plan_pass(const stencil_plan *h, int64_t nx, int64_t ny, int64_t nz, int dty
 }
 
 int encode_map(CUtensorMap *m, const void *ptr, int64_t nx, int64_t ny, int64_t nz, int dtype,
-               int box_w, int box_h)
+               int box_w, int box_h, int64_t pitch = 0)
 {
     auto enc = tensor_map_encoder();
     if (!enc) return STENCIL_ERR_CUDA;
     const int es = elem_bytes(dtype);
     cuuint64_t dims[3] = {static_cast<cuuint64_t>(nx), static_cast<cuuint64_t>(ny),
                           static_cast<cuuint64_t>(nz)};
-    cuuint64_t strides[2] = {static_cast<cuuint64_t>(nx * es), static_cast<cuuint64_t>(nx * ny * es)};
+    if (!pitch) pitch = nx;   // cells from row to row
+    cuuint64_t strides[2] = {static_cast<cuuint64_t>(pitch * es), static_cast<cuuint64_t>(pitch * ny * es)};
     cuuint32_t box[3] = {static_cast<cuuint32_t>(box_w), static_cast<cuuint32_t>(box_h), 1};
     cuuint32_t estr[3] = {1, 1, 1};
     const CUtensorMapDataType dt = dtype == STENCIL_F32    ? CU_TENSOR_MAP_DATA_TYPE_FLOAT32
@@ -554,6 +559,23 @@ int ensure_scratch(stencil_plan *h, size_t bytes)
         h->scratch_bytes = bytes;
         h->scratch_dev = dev;
     }
+    return 0;
+}
+
+// As ensure_scratch for a route that another one can stand in for: *ok is false, with no error, where
+// the memory cannot be had (too little of it, or the stream is being captured).
+int try_scratch(stencil_plan *h, size_t bytes, cudaStream_t st, bool *ok)
+{
+    int dev = 0;
+    CK(cudaGetDevice(&dev));
+    *ok = h->scratch && h->scratch_bytes >= bytes && h->scratch_dev == dev;
+    if (*ok) return 0;
+    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+    CK(cudaStreamIsCapturing(st, &cs));
+    if (cs != cudaStreamCaptureStatusNone) return 0;
+    const int rc = ensure_scratch(h, bytes);
+    if (rc && rc != STENCIL_ERR_OOM) return rc;
+    *ok = rc == 0;
     return 0;
 }
 
@@ -798,30 +820,70 @@ int run_tiles(const stencil_plan *h, const TilePlan &tp, const void *in, void *o
     return 0;
 }
 
+// Rows of any length on kernels that read whole vectors: the padded layout of the grids between
+// the caller's two (pack.cu), rows `pitch` cells apart.
+struct Padded {
+    int64_t pitch = 0;
+    size_t bytes = 0;   // of one grid
+};
+
+Padded padded(int64_t nx, int64_t ny, int64_t nz, int dtype)
+{
+    Padded p;
+    const int64_t m = dtype == STENCIL_F32 ? 4 : 8;
+    p.pitch = (nx + m - 1) / m * m;
+    p.bytes = (static_cast<size_t>(p.pitch * ny * nz) * elem_bytes(dtype) + 255) / 256 * 256;
+    return p;
+}
+
+int launch_pack(const void *in, void *out, int64_t nx, int64_t rows, int dtype, const Padded &p, const DevInfo &dev, cudaStream_t st)
+{
+    int nxi = static_cast<int>(nx), pitch = static_cast<int>(p.pitch);
+    void *args[] = {const_cast<void **>(&in), &out, &nxi, &pitch, &rows};
+    const unsigned blocks = static_cast<unsigned>(std::min<int64_t>((rows + 7) / 8, static_cast<int64_t>(dev.sms) * 16));
+    return launch_pass(stn::pack_fn(elem_bytes(dtype)), dim3(blocks), dim3(32, 8), args, 0, st, true);
+}
+
 // All streaming passes of a run: full passes of the schedule's degree, then the remainder.
-// `scratch` is the second grid of the ping-pong.
+// `scratch` is the second grid of the ping-pong.  rag (rows of any length): scratch holds two padded
+// grids, the first receives a padded copy of the input, and only the last pass writes `out`.
 int run_stream(const stencil_plan *h, const void *in, void *out, void *scratch, int64_t nx, int64_t ny, int64_t nz, int iters,
-               int dtype, const stencil_schedule &s, const DevInfo &dev, cudaStream_t st, double share = 1.0)
+               int dtype, const stencil_schedule &s, const DevInfo &dev, cudaStream_t st, double share = 1.0,
+               const Padded *rag = nullptr)
 {
     const int t = std::max(1, std::min(s.t, iters)), L = (iters + t - 1) / t, t_last = iters - (L - 1) * t;
+    const int64_t nxv = rag ? (nx + 3) / 4 * 4 : nx;   // rows in whole vectors
+    const int kind = rag ? h->kind() | 4 : h->kind();
     Pass full, tail;
-    int rc = plan_pass(h, nx, ny, nz, dtype, t, s, dev, full, false, share);
+    int rc = plan_pass(h, nxv, ny, nz, dtype, t, s, dev, full, false, share, kind);
     if (rc) return rc;
     if (t_last != t) {
-        rc = plan_pass(h, nx, ny, nz, dtype, t_last, s, dev, tail, false, share);
+        rc = plan_pass(h, nxv, ny, nz, dtype, t_last, s, dev, tail, false, share, kind);
         if (rc) return rc;
     }
     const void *src = in;
+    void *pad[2] = {scratch, rag ? static_cast<char *>(scratch) + rag->bytes : nullptr};
+    if (rag) {
+        rc = launch_pack(in, pad[0], nx, ny * nz, dtype, *rag, dev, st);
+        if (rc) return rc;
+        src = pad[0];
+    }
     for (int j = 0; j < L; ++j) {
-        void *dst = ((L - 1 - j) % 2 == 0) ? out : scratch;
+        void *dst = rag ? (j == L - 1 ? out : pad[(j + 1) & 1]) : ((L - 1 - j) % 2 == 0) ? out : scratch;
         Pass &ps = (j == L - 1 && t_last != t) ? tail : full;
         ps.a.in = src;
         ps.a.out = dst;
+        if (rag) {
+            ps.a.nxr = static_cast<int>(nx);
+            ps.a.pin = static_cast<int>(rag->pitch);
+            ps.a.dense = j == L - 1;
+            ps.a.pout = static_cast<int>(j == L - 1 ? nx : rag->pitch);
+        }
         CUtensorMap map;
         std::memset(&map, 0, sizeof(map));
         if (h->dim == 3) {
-            rc = encode_map(&map, src, nx, ny, nz, dtype, 4 * static_cast<int>(ps.block.x) + 2 * ps.padin,
-                            static_cast<int>(ps.block.y) * s.rows_per_thread + 2 * h->r);
+            rc = encode_map(&map, src, nxv, ny, nz, dtype, 4 * static_cast<int>(ps.block.x) + 2 * ps.padin,
+                            static_cast<int>(ps.block.y) * s.rows_per_thread + 2 * h->r, rag ? rag->pitch : 0);
             if (rc) return rc;
         }
         void *args[] = {&map, &ps.a};
@@ -830,6 +892,49 @@ int run_stream(const stencil_plan *h, const void *in, void *out, void *scratch, 
         src = dst;
     }
     return 0;
+}
+
+// Estimated time (us) of a 3D streaming pass of the rule's kernel of degree t, FP32 (16-bit storage
+// runs within 15 % of it): fits to 64^3 .. 512^3 passes, tiles counted whole.
+double stream3_pass_us(int r, int t, int64_t nx, int64_t ny, int64_t nz)
+{
+    static const double fixed[stn::kMaxR + 1] = {0, 3.5, 4.3, 6.7, 8.5, 10, 11}, per_mcell[stn::kMaxR + 1] = {0, 1.17, 1.25, 1.32, 1.7, 2.7, 3.6};
+    const double mcells = static_cast<double>((nx + 63) / 64 * 64) * static_cast<double>((ny + 15) / 16 * 16) * static_cast<double>(nz) * 1e-6;
+    return r == 1 && t >= 2 ? 7.0 + 1.7 * mcells : fixed[r] + per_mcell[r] * mcells;
+}
+
+// One step of the one-step kernel (us): 1.9 us and 0.47 us per term and million cells, fitted to
+// radius 1 (3D) .. 6 (2D).
+double naive_step_us(const stencil_plan *h, double mcells)
+{
+    return 2.5 + mcells * (1.9 + 0.47 * (2 * h->dim * h->r + 1));
+}
+
+// The schedule of the streaming kernels for rows of any length, where the rule's one-step kernel
+// would run: its degree for FP32; one step per pass for 16-bit storage, which that kernel rounds at
+// every step.
+stencil_schedule rag_schedule(stencil_schedule s, int dtype)
+{
+    if (dtype != STENCIL_F32) s.t = 1;
+    return s;
+}
+
+// Whether the rule takes them: 3D (2D grids that are not on register tiles are large) and where the
+// copy and the passes are estimated below the one-step kernel's time.
+bool rag_applicable(const stencil_plan *h, int64_t nx, int64_t ny, int64_t nz, int iters, int dtype, const stencil_schedule &s0)
+{
+    if (s0.kernel != STENCIL_KERNEL_NAIVE || h->checked || h->fault_plane >= 0 || h->tile_mode < 0) return false;
+    if (nx > (1 << 30)) return false;   // the padded row stays an int
+    const stencil_schedule s = rag_schedule(s0, dtype);
+    if (!registry().find(h->dim, h->r, 1, h->dim == 3 ? s.rows_per_thread : 1, dtype, h->kind() | 4)) {
+        if (h->dim == 3 || !registry().find(2, h->r, 1, 1, dtype, h->kind() | 4, 0, 0, s.planes_per_step)) return false;
+    }
+    if (h->dim == 2) return false;
+    if (h->tile_mode > 0) return true;
+    const double mcells = static_cast<double>(nx) * ny * nz * 1e-6;
+    const int t = std::max(1, std::min(s.t, iters));
+    const double us = 2.5 + 0.9 * mcells + (iters + t - 1) / t * stream3_pass_us(h->r, t, nx, ny, nz);
+    return us < iters * naive_step_us(h, mcells);
 }
 
 int run_impl(stencil_plan *h, const void *in, void *out, int64_t nx, int64_t ny, int64_t nz,
@@ -871,13 +976,21 @@ int run_impl(stencil_plan *h, const void *in, void *out, int64_t nx, int64_t ny,
 
     TilePlan tp;
     if (rule && plain && plan_tile(h, nx, ny, dtype, iters, s, *dev, &tp)) {
+        bool ok = true;
         if (iters > tp.t) {
-            rc = ensure_scratch(h, bytes);
+            rc = try_scratch(h, bytes, st, &ok);
             if (rc) return rc;
         }
-        return run_tiles(h, tp, in, out, h->scratch, nx, ny, iters, *dev, st);
+        if (ok) return run_tiles(h, tp, in, out, h->scratch, nx, ny, iters, *dev, st);
     }
 
+    if (rule && plain && rag_applicable(h, nx, ny, nz, iters, dtype, s)) {
+        const Padded p = padded(nx, ny, nz, dtype);
+        bool ok = true;
+        rc = try_scratch(h, 2 * p.bytes, st, &ok);
+        if (rc) return rc;
+        if (ok) return run_stream(h, in, out, h->scratch, nx, ny, nz, iters, dtype, rag_schedule(s, dtype), *dev, st, 1.0, &p);
+    }
     const int t = s.kernel == STENCIL_KERNEL_NAIVE ? 1 : std::max(1, std::min(s.t, iters));
     if (iters > t) {
         rc = ensure_scratch(h, bytes);
@@ -1132,13 +1245,11 @@ bool plan_chains(const stencil_batch_item *items, int n, const DevInfo &dev, std
         }
         if (b.h->checked || b.h->fault_plane >= 0) return false;
         c.tiles = rule && plan_tile(b.h, b.nx, b.ny, b.dtype, b.iters, c.s, dev, &c.tp);
-        // microseconds per million cell updates of the streaming kernels at the rule's degrees
-        static const double us3[stn::kMaxR + 1] = {0, 0.87, 1.25, 1.35, 1.6, 2.5, 3.2};
-        c.us = c.tiles ? c.tp.us
-               : b.h->dim == 2 ? stream_run_us(b.h, b.nx, b.ny, b.dtype, b.iters, c.s)
-                               : us3[b.h->r] * 1e-6 * static_cast<double>(b.nx * b.ny * b.nz) * b.iters;
         const int t = c.tiles ? c.tp.t : std::max(1, std::min(c.s.t, b.iters));
         c.passes = (b.iters + t - 1) / t;
+        c.us = c.tiles ? c.tp.us
+               : b.h->dim == 2 ? stream_run_us(b.h, b.nx, b.ny, b.dtype, b.iters, c.s)
+                               : c.passes * stream3_pass_us(b.h->r, t, b.nx, b.ny, b.nz);
         nodes += c.passes;
         out->push_back(c);
     }
@@ -1636,6 +1747,9 @@ int stencil_run_noalloc(stencil_handle h, const void *in, void *out, int64_t nx,
     if (aligned && plan_tile(h, nx, ny, dtype, iters, s, dev, &tp))
         return run_tiles(h, tp, in, out, nd->scratch, nx, ny, iters, dev, st);
     if (streamable) return run_stream(h, in, out, nd->scratch, nx, ny, nz, iters, dtype, s, dev, st);
+    const Padded p = padded(nx, ny, nz, dtype);
+    if (2 * p.bytes <= kNoAllocScratchBytes && rag_applicable(h, nx, ny, nz, iters, dtype, s))
+        return run_stream(h, in, out, nd->scratch, nx, ny, nz, iters, dtype, rag_schedule(s, dtype), dev, st, 1.0, &p);
     const void *src = in;
     for (int j = 0; j < iters; ++j) {
         void *dst = ((iters - 1 - j) % 2 == 0) ? out : nd->scratch;

@@ -61,6 +61,10 @@ struct SweepArgs {
     int fault_plane;      // test hook: never load this input plane (< 0: off)
     float c[kMaxK];       // coefficients, Eq. 1 order
     alignas(8) float cc[2 * kMaxK];   // each coefficient twice: the operand pairs of the packed two-lane FMAs
+    // RAG kernels (rows of any length): nx is the row rounded up to whole 4-cell vectors, nxr the
+    // row itself.  The input's rows (pitch pin) hold the border cell in the cells between; the
+    // output's (pitch pout) get it there too, unless dense, which stores the cells of the row only.
+    int nxr, pin, pout, dense;
 };
 
 // --------------------------------------------------------------- PTX helpers
@@ -238,6 +242,11 @@ template <> struct Fmt<__half> {
         *reinterpret_cast<uint2 *>(p) = t;
     }
 };
+
+template <typename S> __device__ __forceinline__ S to_storage(float v);
+template <> __device__ __forceinline__ float to_storage<float>(float v) { return v; }
+template <> __device__ __forceinline__ __nv_bfloat16 to_storage<__nv_bfloat16>(float v) { return __float2bfloat16_rn(v); }
+template <> __device__ __forceinline__ __half to_storage<__half>(float v) { return __float2half_rn(v); }
 
 // ------------------------------------------------------ compile-time loops
 template <int I> using IC = std::integral_constant<int, I>;
@@ -468,7 +477,7 @@ __device__ __forceinline__ void mbar_inval(uint32_t bar)
 // one thread block.  Returns false if a bounded wait expired (the device
 // status word is then set).  Leaves the block's shared memory free for the
 // next piece.
-template <int D, int R, int T, int VY, typename S, int TX, int TY, bool SH, bool CHK, int P>
+template <int D, int R, int T, int VY, typename S, int TX, int TY, bool SH, bool CHK, int P, bool RAG>
 __device__ __forceinline__ bool sweep_tile(const CUtensorMap *tmap, const SweepArgs &a, int col, int Z0, int Z1,
                                            unsigned char *smem)
 {
@@ -571,9 +580,21 @@ __device__ __forceinline__ bool sweep_tile(const CUtensorMap *tmap, const SweepA
         const int yl = yl0 + vy;
         ystore[vy] = (D == 2) || (yl >= G::HTY && yl < G::HTY + G::CY && gy0 + yl < a.ny);
     }
-    const int64_t pstride = (D == 3) ? static_cast<int64_t>(a.nx) * a.ny : a.nx;
+    const int pout = RAG ? a.pout : a.nx;              // output row pitch
+    const int64_t pstride = (D == 3) ? static_cast<int64_t>(pout) * a.ny : pout;
     S *const gout = static_cast<S *>(a.out) +
-                    ((D == 3) ? static_cast<int64_t>(gy0 + yl0) * a.nx : 0) + gx;
+                    ((D == 3) ? static_cast<int64_t>(gy0 + yl0) * pout : 0) + gx;
+    // RAG: cells past the row's end in the vector that holds it take its value at every level
+    const bool rag_tile = RAG && gx0 <= a.nxr - 1 && a.nxr - 1 < gx0 + G::BX;   // block-uniform
+    const int rag_cell = a.nxr - 1 - gx;               // own cell of the row's end
+    auto rag_fix = [&](float (&v)[VY][4]) {
+        if (rag_cell >= 0 && rag_cell < 3)
+#pragma unroll
+            for (int vy = 0; vy < VY; ++vy)
+#pragma unroll
+                for (int c = 1; c < 4; ++c) v[vy][c] = c > rag_cell ? v[vy][c - 1] : v[vy][c];
+    };
+    (void)rag_fix;
 
     // A thread whose VY rows cross the grid's top or bottom edge keeps its
     // out-of-grid rows equal to the border row in registers (clamp), since
@@ -680,7 +701,7 @@ __device__ __forceinline__ bool sweep_tile(const CUtensorMap *tmap, const SweepA
         if constexpr (!RPROD) issued_hi = kq;
         if (a.fault_plane >= P * kq && a.fault_plane < P * kq + P) return;   // test hook: never complete
         if constexpr (D == 2) {
-            const int xa = max(ox_in, 0), xb = min(ox_in + PWIN, a.nx);
+            const int xa = max(ox_in, 0), xb = min(ox_in + PWIN, RAG ? a.pin : a.nx);
             uint32_t bytes = xb > xa ? static_cast<uint32_t>((xb - xa) * sizeof(S)) : 0u;
             const int nq = P == 1 ? 1 : min(P, lmax - P * kq + 1);   // planes of this step inside the grid
             if constexpr (CHK) {   // destination inside the slot, source inside the grid, 16-byte units
@@ -696,10 +717,10 @@ __device__ __forceinline__ bool sweep_tile(const CUtensorMap *tmap, const SweepA
             }
             mbar_arrive_expect_tx(bar, bytes * static_cast<uint32_t>(nq));
             if (bytes) {
-                const S *src = static_cast<const S *>(a.in) + static_cast<int64_t>(P * kq) * a.nx + xa;
+                const S *src = static_cast<const S *>(a.in) + static_cast<int64_t>(P * kq) * (RAG ? a.pin : a.nx) + xa;
 #pragma unroll
                 for (int j = 0; j < P; ++j)
-                    if (j < nq) bulk_load(smem_addr(dst0 + j * SLOTIN + (xa - ox_in)), src + static_cast<int64_t>(j) * a.nx, bytes, bar);
+                    if (j < nq) bulk_load(smem_addr(dst0 + j * SLOTIN + (xa - ox_in)), src + static_cast<int64_t>(j) * (RAG ? a.pin : a.nx), bytes, bar);
             }
         } else {
             const int q = kq;   // 3D: one plane per step
@@ -959,6 +980,9 @@ __device__ __forceinline__ bool sweep_tile(const CUtensorMap *tmap, const SweepA
                 res[vy][v] = acc;
             }
         }
+        if constexpr (RAG) {
+            if (rag_tile) rag_fix(res);
+        }
         // the last level's out-of-grid rows are neither stored nor read
         if constexpr (D == 3 && VY > 1 && s < T) {
             if (ytile) clamp_rows(res);
@@ -977,7 +1001,18 @@ __device__ __forceinline__ bool sweep_tile(const CUtensorMap *tmap, const SweepA
                                 continue;
                             }
                         }
-                        Fmt<S>::store4(o + vy * a.nx, res[vy]);
+                        if constexpr (RAG) {
+                            S *w = o + static_cast<int64_t>(vy) * pout;
+                            if (a.dense) {
+#pragma unroll
+                                for (int c = 0; c < 4; ++c)
+                                    if (c <= rag_cell) w[c] = to_storage<S>(res[vy][c]);
+                            } else {
+                                Fmt<S>::store4(w, res[vy]);
+                            }
+                        } else {
+                            Fmt<S>::store4(o + vy * a.nx, res[vy]);
+                        }
                     }
             }
         } else {
@@ -1165,7 +1200,7 @@ __device__ __forceinline__ bool sweep_tile(const CUtensorMap *tmap, const SweepA
 // column b mod (ntx*nty), planes [j*seg, (j+1)*seg) with j = b / (ntx*nty),
 // so blocks running together cover neighbouring tiles of the same planes and
 // share their overlapping halo reads in L2.
-template <int D, int R, int T, int VY, typename S, int TX, int TY, bool SH, bool CHK, int P>
+template <int D, int R, int T, int VY, typename S, int TX, int TY, bool SH, bool CHK, int P, bool RAG = false>
 __device__ __forceinline__ bool sweep_block(const CUtensorMap *tmap, const SweepArgs &a, int b, unsigned char *smem)
 {
     const int cols = a.ntx * a.nty;
@@ -1184,7 +1219,7 @@ __device__ __forceinline__ bool sweep_block(const CUtensorMap *tmap, const Sweep
         const int col = static_cast<int>(w / a.ns);
         const int z0 = static_cast<int>(w - static_cast<int64_t>(col) * a.ns);
         const int z1 = static_cast<int>(min(static_cast<int64_t>(a.ns), z0 + (we - w)));
-        ok = sweep_tile<D, R, T, VY, S, TX, TY, SH, CHK, P>(tmap, a, col, z0, z1, smem);
+        ok = sweep_tile<D, R, T, VY, S, TX, TY, SH, CHK, P, RAG>(tmap, a, col, z0, z1, smem);
         w += z1 - z0;
     }
     return ok;
@@ -1192,13 +1227,13 @@ __device__ __forceinline__ bool sweep_block(const CUtensorMap *tmap, const Sweep
 
 // ------------------------------------------------------------------ kernels
 // One pass over the grid: block b sweeps its planes of the tile columns (sweep_block).
-template <int D, int R, int T, int VY, typename S, int TX, int TY, bool SH, bool CHK, int P>
+template <int D, int R, int T, int VY, typename S, int TX, int TY, bool SH, bool CHK, int P, bool RAG = false>
 __global__ void __launch_bounds__(TX *TY)
     sweep_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_constant__ SweepArgs a)
 {
     extern __shared__ __align__(1024) unsigned char smem[];
     if constexpr (D == 3) grid_dep_launch();
-    sweep_block<D, R, T, VY, S, TX, TY, SH, CHK, P>(&tmap, a, static_cast<int>(blockIdx.x), smem);
+    sweep_block<D, R, T, VY, S, TX, TY, SH, CHK, P, RAG>(&tmap, a, static_cast<int>(blockIdx.x), smem);
 }
 
 // Persistent sweep of many grids of one kernel class, all passes, from a device tile

@@ -85,10 +85,6 @@ template <typename S> __device__ __forceinline__ float cell_in(const S *p);
 template <> __device__ __forceinline__ float cell_in<float>(const float *p) { return *p; }
 template <> __device__ __forceinline__ float cell_in<__nv_bfloat16>(const __nv_bfloat16 *p) { return __bfloat162float(*p); }
 template <> __device__ __forceinline__ float cell_in<__half>(const __half *p) { return __half2float(*p); }
-template <typename S> __device__ __forceinline__ S cell_out(float v);
-template <> __device__ __forceinline__ float cell_out<float>(float v) { return v; }
-template <> __device__ __forceinline__ __nv_bfloat16 cell_out<__nv_bfloat16>(float v) { return __float2bfloat16_rn(v); }
-template <> __device__ __forceinline__ __half cell_out<__half>(float v) { return __float2half_rn(v); }
 
 __device__ __forceinline__ float4 f4(const float (&v)[4]) { return make_float4(v[0], v[1], v[2], v[3]); }
 __device__ __forceinline__ void set4(float (&v)[4], float4 t) { v[0] = t.x; v[1] = t.y; v[2] = t.z; v[3] = t.w; }
@@ -271,7 +267,7 @@ __device__ __forceinline__ void tile2d(const A &a, int blk, float4 *halo)
                     if (y >= r0 && y < r1 && gy0 + v < a.ny) {
 #pragma unroll
                         for (int c = 0; c < 4; ++c)
-                            if (gx + c < a.nx) out[static_cast<int64_t>(v) * a.nx + c] = cell_out<S>(q[v][c]);
+                            if (gx + c < a.nx) out[static_cast<int64_t>(v) * a.nx + c] = to_storage<S>(q[v][c]);
                     }
                 }
             }
