@@ -687,7 +687,7 @@ bool tile_grid(const stn::TileEntry &e, int64_t nx, int64_t ny, int t, TileGrid 
 }
 
 int tile_launch(const stencil_plan *h, const stn::TileEntry &e, int t, int rnd, const void *in, void *out, int64_t nx,
-                int64_t ny, cudaStream_t st)
+                int64_t ny, int64_t pin, int64_t pout, cudaStream_t st)
 {
     TileGrid g;
     if (!tile_grid(e, nx, ny, t, &g)) return STENCIL_ERR_UNSUPPORTED;
@@ -702,8 +702,10 @@ int tile_launch(const stencil_plan *h, const stn::TileEntry &e, int t, int rnd, 
     a.hx = g.hx;
     a.ntx = g.ntx;
     const uintptr_t vec = 4 * elem_bytes(e.dtype);   // bytes of a 4-cell vector
-    a.vin = nx % 4 == 0 && reinterpret_cast<uintptr_t>(in) % vec == 0;
-    a.vout = nx % 4 == 0 && reinterpret_cast<uintptr_t>(out) % vec == 0;
+    a.pin = static_cast<int>(pin);
+    a.pout = static_cast<int>(pout);
+    a.vin = pin % 4 == 0 && reinterpret_cast<uintptr_t>(in) % vec == 0;
+    a.vout = pout % 4 == 0 && reinterpret_cast<uintptr_t>(out) % vec == 0;
     std::memcpy(a.c, h->c, sizeof(float) * h->K);
     void *args[] = {&a};
     return launch_pass(e.fn, dim3(static_cast<unsigned>(g.ntx) * static_cast<unsigned>(g.nty)),
@@ -760,6 +762,14 @@ double stream_run_us(const stencil_plan *h, int64_t nx, int64_t ny, int dtype, i
     return (f.fixed + f.per_mcell * mcells) * (h->shared ? shared[h->r] : 1) * iters / s.t;
 }
 
+// Whether the streaming kernels for rows of any length are compiled for this stencil, at the rows per
+// thread or step of the rule's schedule `s`.
+bool rag_compiled(const stencil_plan *h, int dtype, const stencil_schedule &s)
+{
+    return registry().find(h->dim, h->r, 1, h->dim == 3 ? s.rows_per_thread : 1, dtype, h->kind() | 4, 0, 0,
+                           h->dim == 2 ? s.planes_per_step : 1) != nullptr;
+}
+
 // Whether the rule runs this problem with register tiles, and how: the shape and the steps per
 // pass of the least estimated time, where that is below the streaming passes' (or where the rule
 // would run the one-step kernel: rows that are not whole 16-byte vectors, shared coefficients
@@ -770,7 +780,7 @@ double stream_run_us(const stencil_plan *h, int64_t nx, int64_t ny, int dtype, i
 bool plan_tile(const stencil_plan *h, int64_t nx, int64_t ny, int dtype, int iters, const stencil_schedule &s,
                const DevInfo &dev, TilePlan *tp)
 {
-    if (h->dim != 2 || h->checked || h->fault_plane >= 0 || h->tile_mode < 0) return false;
+    if (h->dim != 2 || h->checked || h->fault_plane >= 0 || h->tile_mode < 0 || h->tile_mode > 1) return false;
     tp->rnd = s.kernel == STENCIL_KERNEL_STREAM && dtype != STENCIL_F32 ? s.t : 1;
     tp->e = nullptr;
     for (const auto &e : tile_entries()) {
@@ -799,25 +809,9 @@ bool plan_tile(const stencil_plan *h, int64_t nx, int64_t ny, int dtype, int ite
     }
     if (!tp->e) return false;
     if (h->tile_mode > 0) return true;
-    return s.kernel != STENCIL_KERNEL_STREAM || tp->us < stream_run_us(h, nx, ny, dtype, iters, s);
-}
-
-// All passes of a run; `scratch` is the second grid of the ping-pong.
-int run_tiles(const stencil_plan *h, const TilePlan &tp, const void *in, void *out, void *scratch, int64_t nx, int64_t ny,
-              int iters, const DevInfo &dev, cudaStream_t st)
-{
-    FnInfo fi;
-    int rc = prepare_fn(tp.e->fn, 32 * tp.e->w, tp.e->smem, dev.max_smem, &fi);
-    if (rc) return rc;
-    const int L = (iters + tp.t - 1) / tp.t, unit = std::min(tp.rnd, iters);
-    const void *src = in;
-    for (int j = 0; j < L; ++j) {
-        void *dst = ((L - 1 - j) % 2 == 0) ? out : scratch;
-        rc = tile_launch(h, *tp.e, tile_steps(iters, L, unit, j), unit, src, dst, nx, ny, st);
-        if (rc) return rc;
-        src = dst;
-    }
-    return 0;
+    if (s.kernel == STENCIL_KERNEL_STREAM) return tp->us < stream_run_us(h, nx, ny, dtype, iters, s);
+    // rows of any length: streaming passes on a padded copy where they are compiled
+    return !rag_compiled(h, dtype, s) || tp->us < 2.5 + 1.3e-6 * static_cast<double>(nx) * ny + stream_run_us(h, nx, ny, dtype, iters, s);
 }
 
 // Rows of any length on kernels that read whole vectors: the padded layout of the grids between
@@ -834,6 +828,29 @@ Padded padded(int64_t nx, int64_t ny, int64_t nz, int dtype)
     p.pitch = (nx + m - 1) / m * m;
     p.bytes = (static_cast<size_t>(p.pitch * ny * nz) * elem_bytes(dtype) + 255) / 256 * 256;
     return p;
+}
+
+// All passes of a run; `scratch` is the second grid of the ping-pong.  rag (rows of any length):
+// scratch holds two padded grids, between which all passes but the first and the last run.
+int run_tiles(const stencil_plan *h, const TilePlan &tp, const void *in, void *out, void *scratch, int64_t nx, int64_t ny,
+              int iters, const DevInfo &dev, cudaStream_t st, const Padded *rag = nullptr)
+{
+    FnInfo fi;
+    int rc = prepare_fn(tp.e->fn, 32 * tp.e->w, tp.e->smem, dev.max_smem, &fi);
+    if (rc) return rc;
+    const int L = (iters + tp.t - 1) / tp.t, unit = std::min(tp.rnd, iters);
+    const void *src = in;
+    int64_t pin = nx;
+    for (int j = 0; j < L; ++j) {
+        void *dst = rag ? (j == L - 1 ? out : static_cast<char *>(scratch) + (j & 1) * rag->bytes)
+                        : ((L - 1 - j) % 2 == 0) ? out : scratch;
+        const int64_t pout = rag && j < L - 1 ? rag->pitch : nx;
+        rc = tile_launch(h, *tp.e, tile_steps(iters, L, unit, j), unit, src, dst, nx, ny, pin, pout, st);
+        if (rc) return rc;
+        src = dst;
+        pin = pout;
+    }
+    return 0;
 }
 
 int launch_pack(const void *in, void *out, int64_t nx, int64_t rows, int dtype, const Padded &p, const DevInfo &dev, cudaStream_t st)
@@ -919,18 +936,15 @@ stencil_schedule rag_schedule(stencil_schedule s, int dtype)
     return s;
 }
 
-// Whether the rule takes them: 3D (2D grids that are not on register tiles are large) and where the
+// Whether the rule takes them: 2D grids that plan_tile left (they are large), and 3D grids where the
 // copy and the passes are estimated below the one-step kernel's time.
 bool rag_applicable(const stencil_plan *h, int64_t nx, int64_t ny, int64_t nz, int iters, int dtype, const stencil_schedule &s0)
 {
     if (s0.kernel != STENCIL_KERNEL_NAIVE || h->checked || h->fault_plane >= 0 || h->tile_mode < 0) return false;
     if (nx > (1 << 30)) return false;   // the padded row stays an int
     const stencil_schedule s = rag_schedule(s0, dtype);
-    if (!registry().find(h->dim, h->r, 1, h->dim == 3 ? s.rows_per_thread : 1, dtype, h->kind() | 4)) {
-        if (h->dim == 3 || !registry().find(2, h->r, 1, 1, dtype, h->kind() | 4, 0, 0, s.planes_per_step)) return false;
-    }
-    if (h->dim == 2) return false;
-    if (h->tile_mode > 0) return true;
+    if (!rag_compiled(h, dtype, s)) return false;
+    if (h->tile_mode > 0 || h->dim == 2) return true;
     const double mcells = static_cast<double>(nx) * ny * nz * 1e-6;
     const int t = std::max(1, std::min(s.t, iters));
     const double us = 2.5 + 0.9 * mcells + (iters + t - 1) / t * stream3_pass_us(h->r, t, nx, ny, nz);
@@ -977,6 +991,12 @@ int run_impl(stencil_plan *h, const void *in, void *out, int64_t nx, int64_t ny,
     TilePlan tp;
     if (rule && plain && plan_tile(h, nx, ny, dtype, iters, s, *dev, &tp)) {
         bool ok = true;
+        if (iters > tp.t && nx % 4) {
+            const Padded p = padded(nx, ny, 1, dtype);
+            rc = try_scratch(h, 2 * p.bytes, st, &ok);
+            if (rc) return rc;
+            if (ok) return run_tiles(h, tp, in, out, h->scratch, nx, ny, iters, *dev, st, &p);
+        }
         if (iters > tp.t) {
             rc = try_scratch(h, bytes, st, &ok);
             if (rc) return rc;
@@ -1697,10 +1717,10 @@ int stencil_set_checked(stencil_handle h, int on)
 
 int stencil_set_tile(stencil_handle h, int mode, int t, int rows)
 {
-    if (!h || mode < -1 || mode > 1 || t < 0 || rows < 0) return STENCIL_ERR_INVALID_ARG;
+    if (!h || mode < -1 || mode > 2 || t < 0 || rows < 0) return STENCIL_ERR_INVALID_ARG;
     h->tile_mode = mode;
-    h->tile_t = mode > 0 ? t : 0;
-    h->tile_v = mode > 0 ? rows : 0;
+    h->tile_t = mode == 1 ? t : 0;
+    h->tile_v = mode == 1 ? rows : 0;
     return STENCIL_OK;
 }
 
@@ -1744,10 +1764,11 @@ int stencil_run_noalloc(stencil_handle h, const void *in, void *out, int64_t nx,
     const bool aligned = (reinterpret_cast<uintptr_t>(in) | reinterpret_cast<uintptr_t>(out)) % 16 == 0;
     const bool streamable = s.kernel == STENCIL_KERNEL_STREAM && aligned;
     TilePlan tp;
-    if (aligned && plan_tile(h, nx, ny, dtype, iters, s, dev, &tp))
-        return run_tiles(h, tp, in, out, nd->scratch, nx, ny, iters, dev, st);
-    if (streamable) return run_stream(h, in, out, nd->scratch, nx, ny, nz, iters, dtype, s, dev, st);
     const Padded p = padded(nx, ny, nz, dtype);
+    const bool pads = nx % 4 && 2 * p.bytes <= kNoAllocScratchBytes;   // two padded grids fit
+    if (aligned && plan_tile(h, nx, ny, dtype, iters, s, dev, &tp))
+        return run_tiles(h, tp, in, out, nd->scratch, nx, ny, iters, dev, st, pads ? &p : nullptr);
+    if (streamable) return run_stream(h, in, out, nd->scratch, nx, ny, nz, iters, dtype, s, dev, st);
     if (2 * p.bytes <= kNoAllocScratchBytes && rag_applicable(h, nx, ny, nz, iters, dtype, s))
         return run_stream(h, in, out, nd->scratch, nx, ny, nz, iters, dtype, rag_schedule(s, dtype), dev, st, 1.0, &p);
     const void *src = in;

