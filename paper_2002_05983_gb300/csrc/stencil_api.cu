@@ -248,9 +248,11 @@ void default_schedule(const stencil_plan *h, int64_t nx, int64_t ny, int64_t nz,
         d.planes_per_step = h->r >= 2 && reg.find(2, h->r, d.t, 1, dtype, h->kind(), 128, 0, 2) ? 2 : 1;
     } else {
         d.t = h->r == 1 ? 2 : 1;
-        // FP32 radius 3 and 4 (one level, packed two-lane arithmetic): 4 rows per thread
-        // measured 670 / 613 against 654 / 591 GCell/s with 2 rows on 512^3
-        const bool four = dtype == STENCIL_F32 && h->kind() == 0 && d.t == 1 && (h->r == 3 || h->r == 4) &&
+        // 4 rows per thread where they measured faster on 512^3 (us per pass, 2 / 4 rows): FP32 radius
+        // 3 204 / 170, 4 213.6 / 212.5, 5 302 / 283; 16-bit radius 2 140 / 131, 3 201 / 175, 4 249 / 236
+        // (FP32 radius 2 168 / 190, 6 380 / 783; 16-bit radius 5 296 / 299, 6 393 / 450)
+        const bool f32 = dtype == STENCIL_F32;
+        const bool four = h->kind() == 0 && d.t == 1 && (f32 ? h->r >= 3 && h->r <= 5 : h->r >= 2 && h->r <= 4) &&
                           reg.find(3, h->r, 1, 4, dtype, 0, 16, 8, 1) != nullptr;
         d.rows_per_thread = four ? 4 : 2;
         d.threads_x = 16;
@@ -915,7 +917,7 @@ int run_stream(const stencil_plan *h, const void *in, void *out, void *scratch, 
 // runs within 15 % of it): fits to 64^3 .. 512^3 passes, tiles counted whole.
 double stream3_pass_us(int r, int t, int64_t nx, int64_t ny, int64_t nz)
 {
-    static const double fixed[stn::kMaxR + 1] = {0, 3.5, 4.3, 6.7, 8.5, 10, 11}, per_mcell[stn::kMaxR + 1] = {0, 1.17, 1.25, 1.32, 1.7, 2.7, 3.6};
+    static const double fixed[stn::kMaxR + 1] = {0, 3.5, 4.3, 6.7, 8.5, 10, 11}, per_mcell[stn::kMaxR + 1] = {0, 1.17, 1.25, 1.32, 1.6, 2.3, 3.0};
     const double mcells = static_cast<double>((nx + 63) / 64 * 64) * static_cast<double>((ny + 15) / 16 * 16) * static_cast<double>(nz) * 1e-6;
     return r == 1 && t >= 2 ? 7.0 + 1.7 * mcells : fixed[r] + per_mcell[r] * mcells;
 }
@@ -1075,10 +1077,10 @@ double analytic_ns(const stencil_plan *h, int64_t nx, int64_t ny, int64_t nz, in
     const double nblk = std::ceil(tiles * ns_axis / s.seg);
     const int P = e->p, VY = e->vy, NV = (R + 3) / 4;
     const double cells = 4.0 * VY * P;                               // per thread, level and step
-    // FP32 instructions per cell: 2*D*r + 1 (both coefficient forms); the 3D FP32 one-level
-    // kernels of radius 3 and 4 run two cells per packed instruction except the x terms of
-    // odd distance: 1/2 for the centre, 3 per even and 4 per odd distance
-    const bool packed = D == 3 && t == 1 && dtype == STENCIL_F32 && !h->shared && (R == 3 || R == 4);
+    // FP32 instructions per cell: 2*D*r + 1 (both coefficient forms); the 3D one-level kernels of
+    // radius 3, FP32 radius 4 and 16-bit radius 5 and 6 run two cells per packed instruction except
+    // the x terms of odd distance: 1/2 for the centre, 3 per even and 4 per odd distance
+    const bool packed = D == 3 && t == 1 && !h->shared && (R == 3 || (dtype == STENCIL_F32 ? R == 4 : R >= 5));
     double fpc = 2.0 * D * R + 1.0;
     if (packed) {
         fpc = 0.5;

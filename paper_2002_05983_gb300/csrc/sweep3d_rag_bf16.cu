@@ -7,9 +7,9 @@ namespace stn {
 namespace {
 const KernelEntry kList[] = {
     STN_ER(3, 1, 1, 2, __nv_bfloat16, 1, false, 1),
-    STN_ER(3, 2, 1, 2, __nv_bfloat16, 1, false, 1),
-    STN_ER(3, 3, 1, 2, __nv_bfloat16, 1, false, 1),
-    STN_ER(3, 4, 1, 2, __nv_bfloat16, 1, false, 1),
+    STN_ER(3, 2, 1, 4, __nv_bfloat16, 1, false, 1),
+    STN_ER(3, 3, 1, 4, __nv_bfloat16, 1, false, 1),
+    STN_ER(3, 4, 1, 4, __nv_bfloat16, 1, false, 1),
     STN_ER(3, 5, 1, 2, __nv_bfloat16, 1, false, 1),
     STN_ER(3, 6, 1, 2, __nv_bfloat16, 1, false, 1)};
 }  // namespace

@@ -7,7 +7,7 @@ namespace stn {
 namespace {
 const KernelEntry kList[] = {
     STN_ER(3, 4, 1, 4, float, 0, false, 1),
-    STN_ER(3, 5, 1, 2, float, 0, false, 1),
+    STN_ER(3, 5, 1, 4, float, 0, false, 1),
     STN_ER(3, 6, 1, 2, float, 0, false, 1),
     STN_ER(3, 3, 1, 2, float, 0, true, 1),
     STN_ER(3, 4, 1, 2, float, 0, true, 1)};

@@ -532,10 +532,12 @@ __device__ __forceinline__ bool sweep_tile(const CUtensorMap *tmap, const SweepA
     // SH: one coefficient per distance, c[0] centre and c[i] for distance i.
     constexpr int K = SH ? 1 + R : 1 + 2 * D * R;
     // Packed two-lane FP32 arithmetic (cells 0,1 and 2,3 of a row in lockstep; bit-identical
-    // to the scalar chain) where it measured faster: 3D FP32 one-level passes of radius 3
-    // (+3 %, coefficient pairs read from the kernel parameters) and 4 (+1.3 %, pairs held in
-    // registers).  Elsewhere its 30-40 extra registers cost more than the issue slots it saves.
-    constexpr bool PK = !SH && D == 3 && T == 1 && F32S && (R == 3 || R == 4);
+    // to the scalar chain) where it measured faster: 3D one-level passes of radius 3 (coefficient
+    // pairs read from the kernel parameters; FP32 +3 %, 16-bit with 4 rows per thread 208 -> 175 us
+    // on 512^3), of radius 4 with FP32 storage (+1.3 %, pairs held in registers) and of radius 5
+    // and 6 with 16-bit storage (321 -> 296 and 401 -> 393 us).  Elsewhere its 30-40 extra registers
+    // cost more than the issue slots it saves.
+    constexpr bool PK = !SH && D == 3 && T == 1 && (R == 3 || (F32S ? R == 4 : R >= 5));
     constexpr bool PKC = R == 3;   // coefficient pairs from the parameters (else registers)
     auto cpair = [&](int k) -> uint64_t {   // coefficient k in both lanes
         if constexpr (PKC) return *reinterpret_cast<const uint64_t *>(&a.cc[2 * k]);
