@@ -755,8 +755,7 @@ double stream_run_us(const stencil_plan *h, int64_t nx, int64_t ny, int dtype, i
     };
     static const Fit f32[stn::kMaxR + 1] = {{}, {38, 1.49}, {22, 1.59}, {22, 1.46}, {28, 1.68}, {64, 2.83}, {120, 4.30}};
     static const Fit b16[stn::kMaxR + 1] = {{}, {43, 1.47}, {24, 1.66}, {45, 2.07}, {33, 1.74}, {66, 2.90}, {125, 4.40}};
-    // one coefficient per distance: compiled with one row per step only
-    static const double shared[stn::kMaxR + 1] = {1, 1, 1.13, 1.18, 1.26, 1, 1};
+    static const double shared[stn::kMaxR + 1] = {1, 1, 1.01, 1.05, 1.03, 1, 1};   // one coefficient per distance
     const Fit &f = (dtype == STENCIL_F32 ? f32 : b16)[h->r];
     const int t = std::max(1, std::min(s.t, iters));
     const int64_t cx = 512 - 2 * round_up((t - 1) * h->r, 4);
