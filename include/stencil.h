@@ -335,11 +335,11 @@ int stencil_set_fault_injection(stencil_handle h, int plane, int timeout_ms);
 /* Which kernels run the library's rule.  2D grids run streaming passes or register tiles (128-cell
  * wide tiles held in registers, any number of steps per pass, rows of any length); grids whose rows
  * are not whole 16-byte vectors run the one-step kernel, tiles or, on a padded copy, streaming
- * passes for rows of any length.  All give the same bits, and stencil_run, stencil_run_ex without a
+ * passes for rows of any length; small 3D grids run one-step passes that march in registers.  All give the same bits, and stencil_run, stencil_run_ex without a
  * schedule and stencil_run_noalloc choose by estimated time; this call is for tests and
- * measurements.  mode 0: choose (the default); -1: never tiles nor padded copies; 1: always where
+ * measurements.  mode 0: choose (the default); -1: the schedule's own kernel only; 1: always where
  * they exist, tiles with at most t steps per pass and `rows` rows per thread (0: chosen); 2: never
- * tiles, always padded copies where their kernels exist.
+ * tiles, always padded copies where their kernels exist; 3: 3D marching passes wherever they can.
  * Errors: INVALID_ARG. */
 int stencil_set_tile(stencil_handle h, int mode, int t, int rows);
 
