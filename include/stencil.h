@@ -94,7 +94,7 @@ typedef struct {
                             of degree t (a remainder pass of another degree runs with
                             its own kernel's depth) */
     int planes_per_step; /* 2D: rows every time level advances per step of the block's loop,
-                            1, 2 (t = 1..5) or 4 (t = 1): the rows of a step share one
+                            1, 2 (t = 1..5) or 4 (t = 1, and radius 3 FP32 at t = 2): the rows of a step share one
                             barrier, one copy wait and the loop's bookkeeping; 3D: 1.  A
                             degree compiled with fewer rows per step runs with the next
                             smaller count that is compiled (4 -> 2 -> 1). */
@@ -176,7 +176,7 @@ int stencil_run_host(stencil_handle h, const void *in_host, void *out_host, int6
  * tuning-cache file (see stencil_tune), else the proposal of the cost model set
  * with stencil_use_cost_model, else the library's rule (2D: radius 1 at t = 4
  * with one row per step, radius 2..4 at t = 3, 2, 2 with two rows per step --
- * 16-bit storage radius 3 at t = 3 --, radius 5, 6 at t = 2; 3D: t = 2 for
+ * 16-bit storage radius 3 at t = 3 --, radius 5, 6 at t = 2 with two rows; 3D: t = 2 for
  * radius 1, else t = 1; 2 rows per thread, 4 for FP32 radius 3 to 5 and 16-bit
  * radius 2 to 4; the
  * one-step kernel for rows that are not whole 16-byte vectors).  Where it is the

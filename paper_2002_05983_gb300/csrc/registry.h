@@ -63,6 +63,7 @@ int list_2d_f32_p2(const KernelEntry **e);
 int list_2d_bf16_p2(const KernelEntry **e);
 int list_2d_f16_p2(const KernelEntry **e);
 int list_2d_p4(const KernelEntry **e);
+int list_2d_p2_wide(const KernelEntry **e);
 int list_rag_f32(const KernelEntry **e);
 int list_rag_f32_wide(const KernelEntry **e);
 int list_rag_bf16(const KernelEntry **e);

@@ -100,7 +100,7 @@ struct Registry {
                            stn::list_3d_bf16_r5, stn::list_3d_bf16_r6, stn::list_2d_f16_r5,
                            stn::list_2d_f16_r6,  stn::list_3d_f16_r5,  stn::list_3d_f16_r6,
                            stn::list_2d_f32sh,   stn::list_3d_f32sh,   stn::list_checked,  stn::list_2d_f32_p2,
-                           stn::list_2d_bf16_p2, stn::list_2d_f16_p2,  stn::list_2d_p4,
+                           stn::list_2d_bf16_p2, stn::list_2d_f16_p2,  stn::list_2d_p4,      stn::list_2d_p2_wide,
                            stn::list_rag_f32,    stn::list_rag_f32_wide, stn::list_rag_bf16,  stn::list_rag_f16,
                            stn::list_rag_2d};
         for (L f : lists) {
@@ -403,6 +403,8 @@ bool chosen_schedule(const stencil_plan *h, int64_t nx, int64_t ny, int64_t nz, 
     h->model_picks.push_back({nx, ny, nz, dtype, gen, pick});
     return false;
 }
+
+void rule_rows(const stencil_plan *h, int64_t nx, int64_t ny, int dtype, stencil_schedule *s);
 
 // Planes per block for 3D grids that the four-wave rule would give fewer than three waves of blocks:
 // as many slabs as fill a whole number of waves, for the number of waves with the least planes on
@@ -755,8 +757,8 @@ double stream_run_us(const stencil_plan *h, int64_t nx, int64_t ny, int dtype, i
     struct Fit {
         double fixed, per_mcell;
     };
-    static const Fit f32[stn::kMaxR + 1] = {{}, {38, 1.49}, {22, 1.59}, {22, 1.46}, {28, 1.68}, {64, 2.83}, {120, 4.30}};
-    static const Fit b16[stn::kMaxR + 1] = {{}, {43, 1.47}, {24, 1.66}, {45, 2.07}, {33, 1.74}, {66, 2.90}, {125, 4.40}};
+    static const Fit f32[stn::kMaxR + 1] = {{}, {38, 1.49}, {22, 1.59}, {31, 1.32}, {28, 1.68}, {64, 2.61}, {101, 3.86}};
+    static const Fit b16[stn::kMaxR + 1] = {{}, {43, 1.47}, {24, 1.66}, {45, 2.07}, {33, 1.74}, {95, 2.57}, {115, 4.30}};
     static const double shared[stn::kMaxR + 1] = {1, 1, 1.01, 1.05, 1.03, 1, 1};   // one coefficient per distance
     const Fit &f = (dtype == STENCIL_F32 ? f32 : b16)[h->r];
     const int t = std::max(1, std::min(s.t, iters));
@@ -1031,6 +1033,17 @@ bool rag_applicable(const stencil_plan *h, int64_t nx, int64_t ny, int64_t nz, i
     return us < iters * naive_step_us(h, mcells);
 }
 
+// Rows per step of the rule's streaming passes where more than the schedule's are faster: four for
+// FP32 radius 3 at t = 2 from 64 million cells on (us a step, two rows / four: 16384^2 206.9 / 192.9,
+// 12000^2 114.3 / 108.4, 8192^2 60.3 / 59.8, 6000^2 36.2 / 37.1; radius 2 and 4 lose: 16384^2 149.5 / 206.1 at
+// t = 3, 238.3 / 241.5).
+void rule_rows(const stencil_plan *h, int64_t nx, int64_t ny, int dtype, stencil_schedule *s)
+{
+    if (h->dim == 2 && h->kind() == 0 && h->r == 3 && dtype == STENCIL_F32 && s->t == 2 && s->planes_per_step == 2 &&
+        nx * ny >= (1LL << 26) && h->tile_mode >= 0 && h->fault_plane < 0)
+        s->planes_per_step = 4;
+}
+
 int run_impl(stencil_plan *h, const void *in, void *out, int64_t nx, int64_t ny, int64_t nz,
              int iters, int dtype, cudaStream_t st, const stencil_schedule *user)
 {
@@ -1109,7 +1122,10 @@ int run_impl(stencil_plan *h, const void *in, void *out, int64_t nx, int64_t ny,
         rc = ensure_scratch(h, bytes);
         if (rc) return rc;
     }
-    if (s.kernel == STENCIL_KERNEL_STREAM) return run_stream(h, in, out, h->scratch, nx, ny, nz, iters, dtype, s, *dev, st);
+    if (s.kernel == STENCIL_KERNEL_STREAM) {
+        if (rule && plain) rule_rows(h, nx, ny, dtype, &s);
+        return run_stream(h, in, out, h->scratch, nx, ny, nz, iters, dtype, s, *dev, st);
+    }
     const void *src = in;
     for (int j = 0; j < iters; ++j) {
         void *dst = ((iters - 1 - j) % 2 == 0) ? out : h->scratch;
@@ -1358,6 +1374,7 @@ bool plan_chains(const stencil_batch_item *items, int n, const DevInfo &dev, std
         }
         if (b.h->checked || b.h->fault_plane >= 0) return false;
         c.tiles = rule && plan_tile(b.h, b.nx, b.ny, b.dtype, b.iters, c.s, dev, &c.tp);
+        if (rule && !c.tiles) rule_rows(b.h, b.nx, b.ny, b.dtype, &c.s);
         const int t = c.tiles ? c.tp.t : std::max(1, std::min(c.s.t, b.iters));
         c.passes = (b.iters + t - 1) / t;
         c.us = c.tiles ? c.tp.us
@@ -1372,11 +1389,11 @@ bool plan_chains(const stencil_batch_item *items, int n, const DevInfo &dev, std
 // One CUDA graph of the grids' chains.  2D passes fill the device, so the 2D grids follow one another
 // on one branch.  A 3D pass of a small grid does not, and cutting it into enough blocks to do so
 // spends most of the planes on halos; every 3D grid has a branch of its own, at high priority, whose
-// passes are cut for six times its share of the batch's work, so the 3D chains run beside the 2D
+// passes are cut for 15 times its share of the batch's work, so the 3D chains run beside the 2D
 // one.  Measured on 16 2D + 8 3D grids, 100 steps: 62 ms as persistent launches per kernel class
-// (a class's blocks hold the SMs until it ends, so a grid of a few tiles runs nearly alone), 46 ms as
-// one chain, 43.5 ms so; cutting for 1.5 / 3 / 12 times the share 54 / 47 / 45 ms, two 2D branches
-// 45 ms; 5 + 3 grids 12.3 -> 7.7 ms, 12 + 2 37.2 -> 21.4, 2 + 8 10.4 -> 5.9.
+// (a class's blocks hold the SMs until it ends, so a grid of a few tiles runs nearly alone), 45.5 ms
+// as one chain, 44.3 ms so; cutting for 1.5 / 4 / 6 / 9 times the share 54 / 46.6 / 45.8 / 46.2 ms,
+// two 2D branches 45.2 ms; 5 + 3 grids 12.3 -> 7.1 ms, 12 + 2 37.2 -> 21.3, 2 + 8 10.4 -> 6.1.
 int build_chains(const stencil_batch_item *items, std::vector<BatchChain> &chains, const DevInfo &dev, BatchEntry *E)
 {
     const int n = static_cast<int>(chains.size());
@@ -1427,7 +1444,7 @@ int build_chains(const stencil_batch_item *items, std::vector<BatchChain> &chain
                 rc = run_tiles(b.h, c->tp, b.in, b.out, scr, b.nx, b.ny, b.iters, dev, br[c->branch]);
             else
                 rc = run_stream(b.h, b.in, b.out, scr, b.nx, b.ny, b.nz, b.iters, b.dtype, c->s, dev, br[c->branch],
-                                b.h->dim == 3 ? std::min(1.0, 6.0 * c->us / total) : 1.0);
+                                b.h->dim == 3 ? std::min(1.0, 15.0 * c->us / total) : 1.0);
         }
         for (int k = 0; k < nb && err == cudaSuccess; ++k) {
             err = cudaEventRecord(ev[k], br[k]);
@@ -1863,7 +1880,10 @@ int stencil_run_noalloc(stencil_handle h, const void *in, void *out, int64_t nx,
         return run_tiles(h, tp, in, out, nd->scratch, nx, ny, iters, dev, st, pads ? &p : nullptr);
     if (aligned && march_applicable(h, nx, ny, nz, dtype, s))
         return run_march(h, in, out, nd->scratch, nx, ny, nz, iters, dtype, dev, st, pads ? &p : nullptr);
-    if (streamable) return run_stream(h, in, out, nd->scratch, nx, ny, nz, iters, dtype, s, dev, st);
+    if (streamable) {
+        rule_rows(h, nx, ny, dtype, &s);
+        return run_stream(h, in, out, nd->scratch, nx, ny, nz, iters, dtype, s, dev, st);
+    }
     if (2 * p.bytes <= kNoAllocScratchBytes && rag_applicable(h, nx, ny, nz, iters, dtype, s))
         return run_stream(h, in, out, nd->scratch, nx, ny, nz, iters, dtype, rag_schedule(s, dtype), dev, st, 1.0, &p);
     const void *src = in;

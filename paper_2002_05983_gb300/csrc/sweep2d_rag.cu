@@ -13,8 +13,8 @@ const KernelEntry kList[] = {
     STN_ER(2, 3, 2, 1, float, 0, false, 2),
     STN_ER(2, 4, 1, 1, float, 0, false, 2),
     STN_ER(2, 4, 2, 1, float, 0, false, 2),
-    STN_ER(2, 5, 1, 1, float, 0, false, 1),
-    STN_ER(2, 5, 2, 1, float, 0, false, 1)};
+    STN_ER(2, 5, 1, 1, float, 0, false, 2),
+    STN_ER(2, 5, 2, 1, float, 0, false, 2)};
 }  // namespace
 int list_rag_2d(const KernelEntry **e)
 {
