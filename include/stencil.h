@@ -296,9 +296,10 @@ typedef struct {
  * and replayed on `stream` by later calls: every grid is a chain of the passes
  * stencil_run would launch; the 2D grids, whose passes fill the device, follow
  * one another, and each 3D grid runs on a parallel branch in passes cut for its
- * part of the device.  Lists of more than 20000 passes, whose graphs would grow
- * too large, and handles with the fault-injection or checked hooks run as
- * persistent launches instead, one per kernel class (dim, radius, dtype,
+ * part of the device.  Lists of 48 grids or more with at least five grids per
+ * (dim, radius, dtype, coefficient form), lists of more than 20000 passes, whose
+ * graphs would grow too large, and handles with the fault-injection, checked or
+ * tile (mode -1) hooks run as persistent launches instead, one per kernel class (dim, radius, dtype,
  * temporal degree, rows per thread or per step) on parallel graph branches:
  * iters / t passes of each grid's tuned or default degree t, then one remainder
  * pass, blocks taking tiles from a device-side queue ordered pass by pass over
@@ -342,6 +343,26 @@ int stencil_set_fault_injection(stencil_handle h, int plane, int timeout_ms);
  * tiles, always padded copies where their kernels exist; 3: 3D marching passes wherever they can.
  * Errors: INVALID_ARG. */
 int stencil_set_tile(stencil_handle h, int mode, int t, int rows);
+
+/* The passes stencil_run would take for this problem when given no schedule (16-byte aligned buffers,
+ * memory available): which kernel, how many launches, the steps of the longest one and, for register
+ * tiles, the rows per thread.  No device work.  Errors: INVALID_ARG, CUDA. */
+typedef enum {
+    STENCIL_PASS_STREAM = 1, /* streaming passes of the schedule */
+    STENCIL_PASS_NAIVE = 2,  /* the one-step kernel */
+    STENCIL_PASS_TILE = 3,   /* 2D register tiles */
+    STENCIL_PASS_MARCH = 4,  /* 3D marching one-step passes */
+    STENCIL_PASS_PADDED = 5  /* streaming passes over a padded copy (one more launch makes it) */
+} stencil_pass_kind;
+typedef struct {
+    int kind;            /* stencil_pass_kind */
+    int t;               /* steps of the longest pass */
+    int launches;        /* kernel launches of the run */
+    int rows_per_thread; /* register tiles and 3D streaming passes, else 0 */
+    int planes_per_step; /* 2D streaming passes, else 0 */
+} stencil_passes;
+int stencil_run_passes(stencil_handle h, int64_t nx, int64_t ny, int64_t nz, int iters, int dtype,
+                       stencil_passes *out);
 
 /* Memory-checker substitute: with on = 1, streaming sweeps on this handle use
  * the bounds-checked kernel instantiations, which test every shared-memory

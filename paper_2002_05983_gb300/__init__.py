@@ -31,7 +31,7 @@ KERNEL_AUTO, KERNEL_STREAM, KERNEL_NAIVE = 0, 1, 2
 # every symbol include/stencil.h declares
 EXPORTS = ("stencil_create", "stencil_create_shared", "stencil_destroy", "stencil_run", "stencil_run_ex", "stencil_run_host",
            "stencil_default_schedule", "stencil_max_t", "stencil_get_device_status",
-           "stencil_set_fault_injection", "stencil_set_checked", "stencil_set_tile", "stencil_run_noalloc", "stencil_run_batched", "stencil_tune",
+           "stencil_set_fault_injection", "stencil_set_checked", "stencil_set_tile", "stencil_run_passes", "stencil_run_noalloc", "stencil_run_batched", "stencil_tune",
            "stencil_resolve_schedule", "stencil_schedule_features", "stencil_model_create", "stencil_model_destroy",
            "stencil_model_train", "stencil_model_predict", "stencil_model_normalization",
            "stencil_model_params", "stencil_model_grad", "stencil_use_cost_model", "stencil_measure_peaks", "stencil_last_cuda_error",
@@ -70,6 +70,15 @@ class Peaks(ctypes.Structure):
                 ("sm_clock_khz", ctypes.c_int)]
 
 
+class Passes(ctypes.Structure):
+    """stencil_passes: the kernel, launches and degree of a run without a schedule."""
+    _fields_ = [("kind", ctypes.c_int), ("t", ctypes.c_int), ("launches", ctypes.c_int),
+                ("rows_per_thread", ctypes.c_int), ("planes_per_step", ctypes.c_int)]
+
+
+PASS_STREAM, PASS_NAIVE, PASS_TILE, PASS_MARCH, PASS_PADDED = 1, 2, 3, 4, 5
+
+
 class Timing(ctypes.Structure):
     """stencil_timing: one candidate schedule with its features and times."""
     _fields_ = [("sched", Schedule), ("features", ctypes.c_float * NFEAT), ("ns_per_cell", ctypes.c_float),
@@ -102,6 +111,7 @@ def _lib():
                 lib.stencil_set_fault_injection.argtypes = [vp, i32, i32]
                 lib.stencil_set_checked.argtypes = [vp, i32]
                 lib.stencil_set_tile.argtypes = [vp, i32, i32, i32]
+                lib.stencil_run_passes.argtypes = [vp, i64, i64, i64, i32, i32, ctypes.POINTER(Passes)]
                 lib.stencil_run_noalloc.argtypes = [vp, vp, vp, i64, i64, i64, i32, i32, vp]
                 lib.stencil_run_batched.argtypes = [ctypes.POINTER(BatchItem), i32, vp]
                 fp = ctypes.POINTER(ctypes.c_float)
@@ -209,6 +219,13 @@ def stencil_set_tile(h, mode: int, t: int = 0, rows: int = 0) -> int:
     """Which kernels run the library's rule (see stencil.h): 0 choose, -1 the schedule's own, 1 tiles and
     padded copies, 2 padded copies."""
     return _check(_lib().stencil_set_tile(h, mode, t, rows), "stencil_set_tile")
+
+
+def stencil_run_passes(h, nx, ny, nz, iters, dtype) -> Passes:
+    """The passes stencil_run would take for this problem when given no schedule."""
+    p = Passes()
+    _check(_lib().stencil_run_passes(h, nx, ny, nz, iters, dtype, ctypes.byref(p)), "stencil_run_passes")
+    return p
 
 
 def stencil_set_fault_injection(h, plane: int, timeout_ms: int = 50) -> int:

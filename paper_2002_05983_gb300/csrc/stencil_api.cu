@@ -11,6 +11,7 @@
 #include <map>
 #include <mutex>
 #include <new>
+#include <set>
 #include <sstream>
 #include <string>
 #include <vector>
@@ -786,6 +787,7 @@ bool plan_tile(const stencil_plan *h, int64_t nx, int64_t ny, int dtype, int ite
                const DevInfo &dev, TilePlan *tp)
 {
     if (h->dim != 2 || h->checked || h->fault_plane >= 0 || h->tile_mode < 0 || h->tile_mode == 2) return false;
+    if (nx > (1 << 30) || ny > (1 << 30)) return false;   // coordinates past the grid stay ints
     tp->rnd = s.kernel == STENCIL_KERNEL_STREAM && dtype != STENCIL_F32 ? s.t : 1;
     tp->e = nullptr;
     for (const auto &e : tile_entries()) {
@@ -1002,9 +1004,9 @@ bool march_applicable(const stencil_plan *h, int64_t nx, int64_t ny, int64_t nz,
     if (h->dim != 3 || h->checked || h->fault_plane >= 0 || h->tile_mode < 0 || h->tile_mode == 2) return false;
     const bool stream = s.kernel == STENCIL_KERNEL_STREAM;
     if (!march_entry(h, dtype, true) || (dtype != STENCIL_F32 && stream && s.t != 1)) return false;
-    if ((nx + 8) * ny > (1LL << 30)) return false;   // offsets within a plane stay ints
+    if (nx > (1 << 30) || (nx + 8) * ny > (1LL << 30) || nz > (1 << 23)) return false;   // offsets within a plane stay ints
     if (h->tile_mode == 3) return true;
-    if (h->tile_mode == 1 || nz > (1 << 23)) return false;
+    if (h->tile_mode == 1) return false;
     const double mcells = static_cast<double>((nx + 63) / 64 * 64) * static_cast<double>((ny + 15) / 16 * 16) * static_cast<double>(nz) * 1e-6;
     return mcells <= (dtype == STENCIL_F32 || h->r == 4 ? 4.0 : 3.0);
 }
@@ -1023,7 +1025,7 @@ stencil_schedule rag_schedule(stencil_schedule s, int dtype)
 bool rag_applicable(const stencil_plan *h, int64_t nx, int64_t ny, int64_t nz, int iters, int dtype, const stencil_schedule &s0)
 {
     if (s0.kernel != STENCIL_KERNEL_NAIVE || h->checked || h->fault_plane >= 0 || h->tile_mode < 0) return false;
-    if (nx > (1 << 30)) return false;   // the padded row stays an int
+    if (nx > (1 << 30) || ny > (1 << 30) || nz > (1 << 30)) return false;   // coordinates past the grid stay ints
     const stencil_schedule s = rag_schedule(s0, dtype);
     if (!rag_compiled(h, dtype, s)) return false;
     if (h->tile_mode > 0 || h->dim == 2) return true;
@@ -1357,14 +1359,21 @@ struct BatchChain {
 // Chains of at most this many launches in all become a graph of ordinary passes; longer lists (and
 // handles with test hooks) keep the persistent launches, whose size does not grow with the steps.
 constexpr int64_t kMaxChainNodes = 20000;
+// So do lists of at least 48 grids with five or more grids per kernel class, where a class's tiles
+// fill the device by themselves: persistent over chained time 1.42 (2 grids per class), 1.34 (2.4),
+// 1.14 (3.2), 1.06 (4.5), 0.93 .. 1.02 (96 grids, 6 per class), 0.94 (64 2D grids, 8 per class), 0.83 (64
+// 3D grids, 8 per class).
+constexpr int kClassGrids = 5, kClassMinGrids = 48;
 
 // Plans every grid's chain; returns false (rc = 0) where the list runs as persistent launches.
 bool plan_chains(const stencil_batch_item *items, int n, const DevInfo &dev, std::vector<BatchChain> *out, int *rc)
 {
     *rc = 0;
     int64_t nodes = 0;
+    std::set<int> classes;   // dimension, radius, storage type, coefficient form
     for (int i = 0; i < n; ++i) {
         const stencil_batch_item &b = items[i];
+        classes.insert(((b.h->dim * 8 + b.h->r) * 4 + b.dtype) * 2 + b.h->shared);
         BatchChain c;
         c.item = i;
         const bool rule = chosen_schedule(b.h, b.nx, b.ny, b.nz, b.dtype, &c.s);
@@ -1372,7 +1381,7 @@ bool plan_chains(const stencil_batch_item *items, int n, const DevInfo &dev, std
             *rc = STENCIL_ERR_UNSUPPORTED;
             return false;
         }
-        if (b.h->checked || b.h->fault_plane >= 0) return false;
+        if (b.h->checked || b.h->fault_plane >= 0 || b.h->tile_mode < 0) return false;
         c.tiles = rule && plan_tile(b.h, b.nx, b.ny, b.dtype, b.iters, c.s, dev, &c.tp);
         if (rule && !c.tiles) rule_rows(b.h, b.nx, b.ny, b.dtype, &c.s);
         const int t = c.tiles ? c.tp.t : std::max(1, std::min(c.s.t, b.iters));
@@ -1383,6 +1392,7 @@ bool plan_chains(const stencil_batch_item *items, int n, const DevInfo &dev, std
         nodes += c.passes;
         out->push_back(c);
     }
+    if (n >= kClassMinGrids && n >= kClassGrids * static_cast<int>(classes.size())) return false;
     return nodes <= kMaxChainNodes;
 }
 
@@ -1831,6 +1841,41 @@ int stencil_set_tile(stencil_handle h, int mode, int t, int rows)
     h->tile_mode = mode;
     h->tile_t = mode == 1 ? t : 0;
     h->tile_v = mode == 1 ? rows : 0;
+    return STENCIL_OK;
+}
+
+int stencil_run_passes(stencil_handle h, int64_t nx, int64_t ny, int64_t nz, int iters, int dtype, stencil_passes *out)
+{
+    if (!h || !out || nx <= 0 || ny <= 0 || nz <= 0 || (h->dim == 2 && nz != 1) || iters < 1 || dtype < STENCIL_F32 ||
+        dtype > STENCIL_F16 || nx > 0x7fffffff || ny > 0x7fffffff || nz > 0x7fffffff)
+        return STENCIL_ERR_INVALID_ARG;
+    DevInfo *dev = nullptr;
+    int rc = device_info(&dev);
+    if (rc) return rc;
+    *out = stencil_passes{};
+    stencil_schedule s;
+    const bool rule = chosen_schedule(h, nx, ny, nz, dtype, &s);
+    TilePlan tp;
+    if (rule && plan_tile(h, nx, ny, dtype, iters, s, *dev, &tp)) {
+        const int L = (iters + tp.t - 1) / tp.t, unit = std::min(tp.rnd, iters);
+        *out = {STENCIL_PASS_TILE, 0, L, tp.e->v, 0};
+        for (int j = 0; j < L; ++j) out->t = std::max(out->t, tile_steps(iters, L, unit, j));
+        return STENCIL_OK;
+    }
+    if (rule && march_applicable(h, nx, ny, nz, dtype, s)) {
+        *out = {STENCIL_PASS_MARCH, 1, iters, 0, 0};
+        return STENCIL_OK;
+    }
+    const bool rag = rule && rag_applicable(h, nx, ny, nz, iters, dtype, s);
+    if (!rag && s.kernel == STENCIL_KERNEL_NAIVE) {
+        *out = {STENCIL_PASS_NAIVE, 1, iters, 0, 0};
+        return STENCIL_OK;
+    }
+    if (rag) s = rag_schedule(s, dtype);
+    else if (rule) rule_rows(h, nx, ny, dtype, &s);
+    const int t = std::max(1, std::min(s.t, iters));
+    *out = {rag ? STENCIL_PASS_PADDED : STENCIL_PASS_STREAM, t, (iters + t - 1) / t + (rag ? 1 : 0),
+            h->dim == 3 ? s.rows_per_thread : 0, h->dim == 2 ? s.planes_per_step : 0};
     return STENCIL_OK;
 }
 

@@ -14,6 +14,8 @@ pytestmark = pytest.mark.gpu
     # many 3D grids (more than the graph's branches), 16-bit storage, single passes and remainders
     [(3, 1 + k % 4, (5 + k, 9 + k, 8 * (1 + k % 5)), 1 + k % 7, ("f32", "bf16", "f16")[k % 3]) for k in range(19)]
     + [(2, 1 + k % 6, (40 + 7 * k, 8 * (3 + k)), 1 + 3 * k, ("f32", "bf16")[k % 2]) for k in range(7)],
+    # 48 grids of three kernel classes: persistent launches
+    [(2 + k % 2, 1 + k % 2, (9 + k, 40) if k % 2 == 0 else (5, 4 + k % 7, 24), 2 + k % 5, "f32") for k in range(48)],
     # 20001 passes of one grid: persistent launches
     [(3, 2, (4, 6, 8), 20001, "f32"), (2, 1, (20, 24), 11, "bf16")],
 ])
