@@ -1494,8 +1494,11 @@ int build_batch(const stencil_batch_item *items, int n, const DevInfo &dev, cuda
         const stencil_batch_item &b = items[i];
         stencil_plan *h = b.h;
         stencil_schedule s;
-        chosen_schedule(h, b.nx, b.ny, b.nz, b.dtype, &s);
+        const bool rule = chosen_schedule(h, b.nx, b.ny, b.nz, b.dtype, &s);
         if (s.kernel != STENCIL_KERNEL_STREAM) return STENCIL_ERR_UNSUPPORTED;
+        // the rule's 4 rows per thread pay on large grids by themselves; the tiles of a batch's mostly
+        // small ones fill less with them, except FP32 radius 3 and 4 (96 grids: 0.152 -> 0.144 s)
+        if (rule && h->dim == 3 && s.rows_per_thread == 4 && (b.dtype != STENCIL_F32 || h->r > 4)) s.rows_per_thread = 2;
         const int t = std::max(1, std::min(s.t, b.iters));
         const int full = b.iters / t, rem = b.iters % t;
         npass[i] = full + (rem ? 1 : 0);
