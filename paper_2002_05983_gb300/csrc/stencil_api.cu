@@ -431,6 +431,14 @@ int64_t whole_wave_seg(int64_t tiles, int64_t ns, int64_t slots, int64_t halo)
     return best;
 }
 
+// Whether a schedule may name `depth` planes loaded ahead for kernel `e`: the compiled number, or, for
+// 3D kernels that take two steps per shifting chunk (3 planes ahead where the ring rounds up to whole
+// chunks), the 2 planes of the one-step form, which schedules kept in files and programs name.
+bool prefetch_ok(const stn::KernelEntry &e, int depth)
+{
+    return depth == e.pf || (depth == 2 && e.dim == 3 && !e.rot && e.u == 2);
+}
+
 // Fill one pass of temporal degree t.  Pointers are set by the caller.
 // batched: tiles of a persistent launch.  share: the part of the device this pass is meant to fill
 // (1: it has the device to itself).  kind: the registry's kernel variant (default the handle's).
@@ -442,14 +450,17 @@ int plan_pass(const stencil_plan *h, int64_t nx, int64_t ny, int64_t nz, int dty
     const int vy = D == 3 ? s.rows_per_thread : 1;
     int pps = D == 2 && s.planes_per_step ? s.planes_per_step : 1;
     const stn::KernelEntry *e = registry().find(D, R, t, vy, dtype, kind, s.threads_x, D == 3 ? s.threads_y : 0, pps);
-    while (!e && pps > 1) {   // a degree compiled with fewer rows per step (e.g. a remainder pass)
-        pps /= 2;
+    // the prefetch depth is a property of the degree-t kernel; a pass of another degree (the
+    // remainder, or fewer iterations than t) runs its own kernel's
+    const bool depth = s.prefetch && t == s.t;
+    // forms with more rows per step beside an older one of the same degree, whose depth may be named
+    auto wider = [&] { return pps == 2 ? h->shared || R >= 5 : pps == 4 && t == 2; };
+    while (pps > 1 && (!e || (depth && wider() && !prefetch_ok(*e, s.prefetch)))) {
+        pps /= 2;   // a degree compiled with fewer rows per step (e.g. a remainder pass)
         e = registry().find(D, R, t, vy, dtype, kind, s.threads_x, 0, pps);
     }
     if (!e) return STENCIL_ERR_UNSUPPORTED;
-    // the prefetch depth is a property of the degree-t kernel; a pass of another degree (the
-    // remainder, or fewer iterations than t) runs its own kernel's
-    if (s.prefetch && t == s.t && s.prefetch != e->pf) return STENCIL_ERR_UNSUPPORTED;
+    if (depth && !prefetch_ok(*e, s.prefetch)) return STENCIL_ERR_UNSUPPORTED;
     if (e->smem > static_cast<size_t>(dev.max_smem)) return STENCIL_ERR_UNSUPPORTED;
     FnInfo fi;
     int rc = prepare_fn(e->fn, e->tx * e->ty, e->smem, dev.max_smem, &fi);
