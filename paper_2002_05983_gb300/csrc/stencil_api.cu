@@ -407,14 +407,19 @@ bool chosen_schedule(const stencil_plan *h, int64_t nx, int64_t ny, int64_t nz, 
 
 void rule_rows(const stencil_plan *h, int64_t nx, int64_t ny, int dtype, stencil_schedule *s);
 
-// Planes per block for 3D grids that the four-wave rule would give fewer than three waves of blocks:
-// as many slabs as fill a whole number of waves, for the number of waves with the least planes on
-// the critical path (waves x (planes + halo planes)).  A block walks its planes one after another
-// at 0.3-0.6 us each however empty the device is, so a small grid wants one wave of short blocks,
-// and a partly filled last wave costs a whole one.  Over 130 measured (kernel, shape) pairs it
-// picks within 1.6 % of the best segment on average (22 % at most); four waves of at least 64
-// planes, the rule for larger grids, was 160 % off there (96^3 radius 2: 26.4 against 5.9 us per
-// pass, 256^3 radius 4: 72.7 against 37.9) and 0-4 % off on 512^3, where whole waves lose up to 8 %.
+// Planes per block of 3D passes whose tiles leave the device partly empty: as many slabs as fill a whole
+// number of waves, for the number of waves with the least planes on the critical path (waves x (planes
+// + halo planes)).  A block walks its planes one after another at 0.3-0.6 us each however empty the
+// device is, so a small grid wants one wave of short blocks, and a partly filled last wave costs a
+// whole one.  Against four waves of at least 64 planes, the rule for larger grids (96^3 radius 2: 26.4 ->
+// 5.9 us per pass, 256^3 radius 4: 72.7 -> 37.9), over 630 (kernel, shape) pairs, time with whole waves
+// over time without:
+//   the library's own degree and rows per thread, below three waves: 153 of 159 at or below 1.01, six up
+//   to 1.13 (radius 1, 5 and 6), none slower than before the other changes to these kernels;
+//   other degrees and rows, below half a wave: 0.10-0.72, 0.29 on average;
+//   these from half a wave to three: 0.47-1.24, with losses scattered over all of that range (radius 1 t = 3
+//   1024 x 300 x 100 91.9 -> 112.9 us a pass, radius 2 with 4 rows 384^3 78.2 -> 87.3, radius 3 t = 2 256^3
+//   135.7 -> 150.4, 16-bit radius 5 448^3 217 -> 245), so they keep four waves there.
 int64_t whole_wave_seg(int64_t tiles, int64_t ns, int64_t slots, int64_t halo)
 {
     int64_t best = ns, cost = INT64_MAX;
@@ -429,6 +434,14 @@ int64_t whole_wave_seg(int64_t tiles, int64_t ns, int64_t slots, int64_t halo)
         if (slabs == ns) break;
     }
     return best;
+}
+
+// Whether a 3D pass has the degree and rows per thread of the library's rule (rows of any length: always).
+bool rule_pass(const stencil_plan *h, int64_t nx, int64_t ny, int64_t nz, int dtype, int t, int rows, int kind)
+{
+    stencil_schedule d;
+    default_schedule(h, nx, ny, nz, dtype, &d);
+    return (kind & 4) || (t == d.t && rows == d.rows_per_thread);
 }
 
 // Whether a schedule may name `depth` planes loaded ahead for kernel `e`: the compiled number, or, for
@@ -491,7 +504,8 @@ int plan_pass(const stencil_plan *h, int64_t nx, int64_t ny, int64_t nz, int dty
             // >= 4 waves (dynamic balance of edge tiles), segments long against the fill
             const int64_t want = (4 * slots + tiles - 1) / tiles;
             seg = std::max<int64_t>((ns + want - 1) / want, minseg);
-            if (D == 3 && !batched && (share < 1 || tiles * ((ns + seg - 1) / seg) < 3 * slots))
+            const double waves = static_cast<double>(tiles * ((ns + seg - 1) / seg)) / static_cast<double>(slots);
+            if (D == 3 && !batched && (share < 1 || waves < (rule_pass(h, nx, ny, nz, dtype, t, vy, kind) ? 3.0 : 0.5)))
                 seg = whole_wave_seg(tiles, ns, std::max<int64_t>(1, static_cast<int64_t>(static_cast<double>(slots) * share)), 2 * R * t);
         } else if (batched) {
             // other grids fill the device: segments long against the pipeline fill
