@@ -293,13 +293,13 @@ typedef struct {
  * together (not in the paper; a serving-style batch of the paper's sweep).
  * Results equal stencil_run's bit for bit.  The list becomes one CUDA graph that
  * is cached for this exact item list (same pointers, sizes, handles, schedules)
- * and replayed on `stream` by later calls: every grid is a chain of the passes
- * stencil_run would launch; the 2D grids, whose passes fill the device, follow
- * one another, and each 3D grid runs on a parallel branch in passes cut for its
- * part of the device.  Lists of 48 grids or more with at least five grids per
- * (dim, radius, dtype, coefficient form), lists of more than 20000 passes, whose
+ * and replayed on `stream` by later calls.  Lists with fewer than three grids per
+ * (dim, radius, dtype, coefficient form) become chains of passes: the 2D grids, on
+ * register tiles or streaming passes as in stencil_run, follow one another, and
+ * each 3D grid runs on a parallel branch in streaming passes cut for its part of
+ * the device.  Lists with more, lists of more than 20000 passes, whose
  * graphs would grow too large, and handles with the fault-injection, checked or
- * tile (mode -1) hooks run as persistent launches instead, one per kernel class (dim, radius, dtype,
+ * tile (mode -1) hooks run as persistent launches, one per kernel class (dim, radius, dtype,
  * temporal degree, rows per thread or per step) on parallel graph branches:
  * iters / t passes of each grid's tuned or default degree t, then one remainder
  * pass, blocks taking tiles from a device-side queue ordered pass by pass over

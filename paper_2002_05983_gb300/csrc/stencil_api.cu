@@ -18,6 +18,7 @@
 
 #include <cudaTypedefs.h>
 
+#include "batch_rule.h"
 #include "march.h"
 #include "march_kernel.cuh"
 #include "naive.h"
@@ -1381,15 +1382,6 @@ struct BatchChain {
     int branch = 0;
 };
 
-// Chains of at most this many launches in all become a graph of ordinary passes; longer lists (and
-// handles with test hooks) keep the persistent launches, whose size does not grow with the steps.
-constexpr int64_t kMaxChainNodes = 20000;
-// So do lists of at least 48 grids with five or more grids per kernel class, where a class's tiles
-// fill the device by themselves: persistent over chained time 1.42 (2 grids per class), 1.34 (2.4),
-// 1.14 (3.2), 1.06 (4.5), 0.93 .. 1.02 (96 grids, 6 per class), 0.94 (64 2D grids, 8 per class), 0.83 (64
-// 3D grids, 8 per class).
-constexpr int kClassGrids = 5, kClassMinGrids = 48;
-
 // Plans every grid's chain; returns false (rc = 0) where the list runs as persistent launches.
 bool plan_chains(const stencil_batch_item *items, int n, const DevInfo &dev, std::vector<BatchChain> *out, int *rc)
 {
@@ -1417,8 +1409,7 @@ bool plan_chains(const stencil_batch_item *items, int n, const DevInfo &dev, std
         nodes += c.passes;
         out->push_back(c);
     }
-    if (n >= kClassMinGrids && n >= kClassGrids * static_cast<int>(classes.size())) return false;
-    return nodes <= kMaxChainNodes;
+    return stn::batch_as_chains(n, static_cast<int>(classes.size()), nodes);
 }
 
 // One CUDA graph of the grids' chains.  2D passes fill the device, so the 2D grids follow one another
