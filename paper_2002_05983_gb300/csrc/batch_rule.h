@@ -1,5 +1,6 @@
 // Which form a batch takes (host code without CUDA types).
 #pragma once
+#include <algorithm>
 #include <cstdint>
 
 namespace stn {
@@ -21,6 +22,17 @@ constexpr int kClassGrids = 3;
 inline bool batch_as_chains(int grids, int classes, int64_t passes)
 {
     return grids < kClassGrids * classes && passes <= kMaxChainNodes;
+}
+
+// Blocks of a persistent class: at most the resident slots, the tiles of all its passes, and twice the
+// tiles of one pass of every grid.  At most one pass of a grid can run at a time, so more blocks would
+// only hold registers and shared memory while they wait, which the classes beside this one need (64
+// grids of 64^3, radius 1 to 4: 12.4-15.4 -> 7.9 ms); once the pass's tiles alone are allowed, blocks waiting for a
+// slow grid keep ready tiles of the next pass from being taken (64 of 1024^2: 14.1 ms with every slot or
+// twice the tiles, 15.6 with the tiles).  Over 147 lists 0.90 of the time with every slot, none slower.
+inline int64_t batch_blocks(int64_t tiles, int64_t pass_tiles, int64_t slots)
+{
+    return std::min(std::min(tiles, 2 * pass_tiles), slots);
 }
 
 }  // namespace stn

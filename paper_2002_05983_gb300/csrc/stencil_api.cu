@@ -1554,7 +1554,7 @@ int build_batch(const stencil_batch_item *items, int n, const DevInfo &dev, cuda
             std::vector<CUtensorMap> maps;
             std::vector<stn::BatchTask> tasks;
             std::vector<int> last_task(n, -1);
-            int total = 0, fault_task = -1, timeout = 2000;
+            int total = 0, first = 0, fault_task = -1, timeout = 2000;
             for (const Pass1 *x : mine) {
                 const stencil_batch_item &b = items[x->item];
                 const int L = npass[x->item], p = x->pass;
@@ -1578,6 +1578,7 @@ int build_batch(const stencil_batch_item *items, int n, const DevInfo &dev, cuda
                 tk.ntiles = static_cast<int>(x->ps.grid.x);
                 tk.first = total;
                 total += tk.ntiles;
+                if (tk.prev < 0) first += tk.ntiles;   // tiles of every grid's first pass
                 if (b.h->fault_plane == p && fault_task < 0) fault_task = static_cast<int>(tasks.size());
                 timeout = b.h->timeout_ms;
                 last_task[x->item] = static_cast<int>(tasks.size());
@@ -1594,7 +1595,7 @@ int build_batch(const stencil_batch_item *items, int n, const DevInfo &dev, cuda
             if (rc) return rc;
             const int occ = fi.occ;
             if (occ < 1) return STENCIL_ERR_UNSUPPORTED;
-            c.grid = dim3(static_cast<unsigned>(std::min<int64_t>(total, static_cast<int64_t>(dev.sms) * occ)));
+            c.grid = dim3(static_cast<unsigned>(stn::batch_blocks(total, first, static_cast<int64_t>(dev.sms) * occ)));
             const int nt = static_cast<int>(tasks.size());
             CK(cudaMalloc(&c.dev_args, sizeof(stn::SweepArgs) * nt));
             CK(cudaMalloc(&c.dev_maps, sizeof(CUtensorMap) * nt));
