@@ -23,6 +23,7 @@
 #include "march_kernel.cuh"
 #include "naive.h"
 #include "pack.h"
+#include "pass_rule.h"
 #include "registry.h"
 #include "stencil.h"
 #include "sweep_kernel.cuh"
@@ -220,6 +221,7 @@ struct Pass {
     int occ = 0;   // resident blocks per SM
     int regs = 0;  // registers per thread of the kernel
     int padin = 0; // input-plane x padding per side: 3D tensor-map box width 4*block.x + 2*padin
+    bool dependent = false;   // launched as a programmatic dependent of the work before it
     dim3 grid, block;
     size_t smem = 0;
     stn::SweepArgs a{};
@@ -500,13 +502,15 @@ int plan_pass(const stencil_plan *h, int64_t nx, int64_t ny, int64_t nz, int dty
     const bool flat = D == 2 && (body > 400 || t >= 5);
     const int64_t W = tiles * ns;
     int64_t seg = s.seg;
+    bool whole = false;   // the segment fills whole waves
     if (seg <= 0) {
         if (!flat) {
             // >= 4 waves (dynamic balance of edge tiles), segments long against the fill
             const int64_t want = (4 * slots + tiles - 1) / tiles;
             seg = std::max<int64_t>((ns + want - 1) / want, minseg);
             const double waves = static_cast<double>(tiles * ((ns + seg - 1) / seg)) / static_cast<double>(slots);
-            if (D == 3 && !batched && (share < 1 || waves < (rule_pass(h, nx, ny, nz, dtype, t, vy, kind) ? 3.0 : 0.5)))
+            whole = D == 3 && !batched && (share < 1 || waves < (rule_pass(h, nx, ny, nz, dtype, t, vy, kind) ? 3.0 : 0.5));
+            if (whole)
                 seg = whole_wave_seg(tiles, ns, std::max<int64_t>(1, static_cast<int64_t>(static_cast<double>(slots) * share)), 2 * R * t);
         } else if (batched) {
             // other grids fill the device: segments long against the pipeline fill
@@ -531,6 +535,7 @@ int plan_pass(const stencil_plan *h, int64_t nx, int64_t ny, int64_t nz, int dty
     ps.block = dim3(e->tx, e->ty);
     ps.smem = e->smem;
     ps.padin = e->padin;
+    ps.dependent = D == 3 && stn::dependent_pass(whole, nblk, slots);
     stn::SweepArgs &a = ps.a;
     a.nx = static_cast<int>(nx);
     a.ny = static_cast<int>(ny);
@@ -937,7 +942,7 @@ int run_stream(const stencil_plan *h, const void *in, void *out, void *scratch, 
             if (rc) return rc;
         }
         void *args[] = {&map, &ps.a};
-        rc = launch_pass(ps.fn, ps.grid, ps.block, args, ps.smem, st, h->dim == 3);
+        rc = launch_pass(ps.fn, ps.grid, ps.block, args, ps.smem, st, ps.dependent);
         if (rc) return rc;
         src = dst;
     }
