@@ -417,8 +417,10 @@ void rule_rows(const stencil_plan *h, int64_t nx, int64_t ny, int dtype, stencil
 // whole one.  Against four waves of at least 64 planes, the rule for larger grids (96^3 radius 2: 26.4 ->
 // 5.9 us per pass, 256^3 radius 4: 72.7 -> 37.9), over 630 (kernel, shape) pairs, time with whole waves
 // over time without:
-//   the library's own degree and rows per thread, below three waves: 153 of 159 at or below 1.01, six up
-//   to 1.13 (radius 1, 5 and 6), none slower than before the other changes to these kernels;
+//   the library's own degree and rows per thread at radius 2 to 6, below three waves: 0.5-1.02, one pair
+//   1.13 (16-bit radius 5 448^3, 0.96 of its time before the other changes to that kernel);
+//   radius 1 (t = 2), below one wave: 0.2-1.0; from there on 0.96-1.08 without a pattern (154 x 653 x 368
+//   34.7 -> 37.7 us a step, 400^3 60.1 -> 63.7, 448^3 0.96 of it), so it keeps four waves there;
 //   other degrees and rows, below half a wave: 0.10-0.72, 0.29 on average;
 //   these from half a wave to three: 0.47-1.24, with losses scattered over all of that range (radius 1 t = 3
 //   1024 x 300 x 100 91.9 -> 112.9 us a pass, radius 2 with 4 rows 384^3 78.2 -> 87.3, radius 3 t = 2 256^3
@@ -509,7 +511,7 @@ int plan_pass(const stencil_plan *h, int64_t nx, int64_t ny, int64_t nz, int dty
             const int64_t want = (4 * slots + tiles - 1) / tiles;
             seg = std::max<int64_t>((ns + want - 1) / want, minseg);
             const double waves = static_cast<double>(tiles * ((ns + seg - 1) / seg)) / static_cast<double>(slots);
-            whole = D == 3 && !batched && (share < 1 || waves < (rule_pass(h, nx, ny, nz, dtype, t, vy, kind) ? 3.0 : 0.5));
+            whole = D == 3 && !batched && (share < 1 || waves < (!rule_pass(h, nx, ny, nz, dtype, t, vy, kind) ? 0.5 : R == 1 ? 1.0 : 3.0));
             if (whole)
                 seg = whole_wave_seg(tiles, ns, std::max<int64_t>(1, static_cast<int64_t>(static_cast<double>(slots) * share)), 2 * R * t);
         } else if (batched) {
