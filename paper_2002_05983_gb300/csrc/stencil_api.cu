@@ -944,7 +944,9 @@ int run_stream(const stencil_plan *h, const void *in, void *out, void *scratch, 
             if (rc) return rc;
         }
         void *args[] = {&map, &ps.a};
-        rc = launch_pass(ps.fn, ps.grid, ps.block, args, ps.smem, st, ps.dependent);
+        // after another kind of pass (the run's first and its remainder pass) slots may be free unevenly
+        const bool like = j > 0 ? j < L - 1 || t_last == t : rag != nullptr;
+        rc = launch_pass(ps.fn, ps.grid, ps.block, args, ps.smem, st, ps.dependent && like);
         if (rc) return rc;
         src = dst;
     }

@@ -25,4 +25,6 @@ def test_dependent_passes(tmp_path):
     assert [bool(int(g)) for g in got] == [w for *_, w in PASSES]
     with open(os.path.join(CSRC, "stencil_api.cu")) as fh:
         api = fh.read()
-    assert "st, ps.dependent)" in api and "st, h->dim == 3)" not in api   # the streaming launch uses the rule
+    assert "st, ps.dependent && like)" in api and "st, h->dim == 3)" not in api   # the streaming launch uses the rule
+    # and not beside another kind of pass
+    assert "const bool like = j > 0 ? j < L - 1 || t_last == t : rag != nullptr;" in api
