@@ -177,8 +177,9 @@ int stencil_run_host(stencil_handle h, const void *in_host, void *out_host, int6
  * with stencil_use_cost_model, else the library's rule (2D: radius 1 at t = 4
  * with one row per step, radius 2..4 at t = 3, 2, 2 with two rows per step --
  * 16-bit storage radius 3 at t = 3 --, radius 5, 6 at t = 2 with two rows; 3D: t = 2 for
- * radius 1, else t = 1; 2 rows per thread, 4 for FP32 radius 3 to 5 and 16-bit
- * radius 2 to 4; the
+ * radius 1, else t = 1; 2 rows per thread, 4 for radius 3, FP32 radius 4 and,
+ * where ny rounds up to whole 32-row tiles at most 3 % further than to 16-row
+ * ones, FP32 radius 5 and 16-bit radius 2 and 4; the
  * one-step kernel for rows that are not whole 16-byte vectors).  Where it is the
  * library's rule, runs may take the same steps on other kernels
  * (stencil_set_tile), with other passes and the same bits: FP32 results do not

@@ -235,7 +235,6 @@ bool stream_applicable(int dtype, int64_t nx)
 void default_schedule(const stencil_plan *h, int64_t nx, int64_t ny, int64_t nz, int dtype,
                       stencil_schedule *s)
 {
-    (void)ny;
     (void)nz;
     const Registry &reg = registry();
     stencil_schedule d{};
@@ -257,8 +256,14 @@ void default_schedule(const stencil_plan *h, int64_t nx, int64_t ny, int64_t nz,
         // 4 rows per thread where they measured faster on 512^3 (us per pass, 2 / 4 rows): FP32 radius
         // 3 204 / 170, 4 213.6 / 212.5, 5 302 / 283; 16-bit radius 2 140 / 131, 3 201 / 175, 4 249 / 236
         // (FP32 radius 2 168 / 190, 6 380 / 783; 16-bit radius 5 296 / 299, 6 393 / 450)
+        // Tiles of 4 rows are 32 rows high, of 2 rows 16: where the gain is 7 % or less, 4 rows only on grids
+        // whose height they round up at most 3 % further (4 / 2 rows, us a step: 1024 x 300 x 100, 5 % further,
+        // FP16 radius 2 42.6 / 40.8, BF16 radius 4 78.2 / 65.6; 480 x 295 x 226 FP32 radius 5 100 / 80.7; 616 x 357 x
+        // 525 FP16 radius 2, 4 % further, 126.7 / 129.8)
         const bool f32 = dtype == STENCIL_F32;
-        const bool four = h->kind() == 0 && d.t == 1 && (f32 ? h->r >= 3 && h->r <= 5 : h->r >= 2 && h->r <= 4) &&
+        const int64_t up4 = (ny + 31) / 32 * 32, up2 = (ny + 15) / 16 * 16;
+        const bool fits = h->r == 3 || (f32 && h->r == 4) || d.kernel == STENCIL_KERNEL_NAIVE || 100 * up4 <= 103 * up2;
+        const bool four = fits && h->kind() == 0 && d.t == 1 && (f32 ? h->r >= 3 && h->r <= 5 : h->r >= 2 && h->r <= 4) &&
                           reg.find(3, h->r, 1, 4, dtype, 0, 16, 8, 1) != nullptr;
         d.rows_per_thread = four ? 4 : 2;
         d.threads_x = 16;
