@@ -413,8 +413,6 @@ bool chosen_schedule(const stencil_plan *h, int64_t nx, int64_t ny, int64_t nz, 
     return false;
 }
 
-void rule_rows(const stencil_plan *h, int64_t nx, int64_t ny, int dtype, stencil_schedule *s);
-
 // Planes per block of 3D passes whose tiles leave the device partly empty: as many slabs as fill a whole
 // number of waves, for the number of waves with the least planes on the critical path (waves x (planes
 // + halo planes)).  A block walks its planes one after another at 0.3-0.6 us each however empty the
@@ -906,23 +904,38 @@ int launch_pack(const void *in, void *out, int64_t nx, int64_t rows, int dtype, 
     return launch_pass(stn::pack_fn(elem_bytes(dtype)), dim3(blocks), dim3(32, 8), args, 0, st, true);
 }
 
+// Rows per step of a pass of degree t of the rule's schedule where more than the schedule's are faster: four
+// for FP32 radius 3 at t = 2 from 64 million cells on (us a step, two rows / four: 16384^2 206.9 / 192.9,
+// 12000^2 114.3 / 108.4, 8192^2 60.3 / 59.8, 6000^2 36.2 / 37.1; radius 2 and 4 lose: 16384^2 149.5 / 206.1 at
+// t = 3, 238.3 / 241.5; so does a single step, the remainder of an odd number: 8192^2 94.9 / 99.5, 12000^2
+// 186.5 / 193.7).
+void rule_rows(const stencil_plan *h, int64_t nx, int64_t ny, int dtype, int t, stencil_schedule *s)
+{
+    if (h->dim == 2 && h->kind() == 0 && h->r == 3 && dtype == STENCIL_F32 && t == 2 && s->planes_per_step == 2 &&
+        nx * ny >= (1LL << 26) && h->tile_mode >= 0 && h->fault_plane < 0)
+        s->planes_per_step = 4;
+}
+
 // All streaming passes of a run: full passes of the schedule's degree, then the remainder.
 // `scratch` is the second grid of the ping-pong.  rag (rows of any length): scratch holds two padded
-// grids, the first receives a padded copy of the input, and only the last pass writes `out`.
+// grids, the first receives a padded copy of the input, and only the last pass writes `out`.  rule: `s` is
+// the library's rule, not a caller's or a stored schedule.
 int run_stream(const stencil_plan *h, const void *in, void *out, void *scratch, int64_t nx, int64_t ny, int64_t nz, int iters,
-               int dtype, const stencil_schedule &s, const DevInfo &dev, cudaStream_t st, double share = 1.0,
+               int dtype, stencil_schedule s, const DevInfo &dev, cudaStream_t st, bool rule, double share = 1.0,
                const Padded *rag = nullptr)
 {
     const int t = std::max(1, std::min(s.t, iters)), L = (iters + t - 1) / t, t_last = iters - (L - 1) * t;
     const int64_t nxv = rag ? (nx + 3) / 4 * 4 : nx;   // rows in whole vectors
     const int kind = rag ? h->kind() | 4 : h->kind();
     Pass full, tail;
-    int rc = plan_pass(h, nxv, ny, nz, dtype, t, s, dev, full, false, share, kind);
-    if (rc) return rc;
+    int rc = 0;
     if (t_last != t) {
         rc = plan_pass(h, nxv, ny, nz, dtype, t_last, s, dev, tail, false, share, kind);
         if (rc) return rc;
     }
+    if (rule && !rag) rule_rows(h, nx, ny, dtype, t, &s);
+    rc = plan_pass(h, nxv, ny, nz, dtype, t, s, dev, full, false, share, kind);
+    if (rc) return rc;
     const void *src = in;
     void *pad[2] = {scratch, rag ? static_cast<char *>(scratch) + rag->bytes : nullptr};
     if (rag) {
@@ -1075,17 +1088,6 @@ bool rag_applicable(const stencil_plan *h, int64_t nx, int64_t ny, int64_t nz, i
     return us < iters * naive_step_us(h, mcells);
 }
 
-// Rows per step of the rule's streaming passes where more than the schedule's are faster: four for
-// FP32 radius 3 at t = 2 from 64 million cells on (us a step, two rows / four: 16384^2 206.9 / 192.9,
-// 12000^2 114.3 / 108.4, 8192^2 60.3 / 59.8, 6000^2 36.2 / 37.1; radius 2 and 4 lose: 16384^2 149.5 / 206.1 at
-// t = 3, 238.3 / 241.5).
-void rule_rows(const stencil_plan *h, int64_t nx, int64_t ny, int dtype, stencil_schedule *s)
-{
-    if (h->dim == 2 && h->kind() == 0 && h->r == 3 && dtype == STENCIL_F32 && s->t == 2 && s->planes_per_step == 2 &&
-        nx * ny >= (1LL << 26) && h->tile_mode >= 0 && h->fault_plane < 0)
-        s->planes_per_step = 4;
-}
-
 int run_impl(stencil_plan *h, const void *in, void *out, int64_t nx, int64_t ny, int64_t nz,
              int iters, int dtype, cudaStream_t st, const stencil_schedule *user)
 {
@@ -1157,17 +1159,15 @@ int run_impl(stencil_plan *h, const void *in, void *out, int64_t nx, int64_t ny,
         bool ok = true;
         rc = try_scratch(h, 2 * p.bytes, st, &ok);
         if (rc) return rc;
-        if (ok) return run_stream(h, in, out, h->scratch, nx, ny, nz, iters, dtype, rag_schedule(s, dtype), *dev, st, 1.0, &p);
+        if (ok) return run_stream(h, in, out, h->scratch, nx, ny, nz, iters, dtype, rag_schedule(s, dtype), *dev, st, true, 1.0, &p);
     }
     const int t = s.kernel == STENCIL_KERNEL_NAIVE ? 1 : std::max(1, std::min(s.t, iters));
     if (iters > t) {
         rc = ensure_scratch(h, bytes);
         if (rc) return rc;
     }
-    if (s.kernel == STENCIL_KERNEL_STREAM) {
-        if (rule && plain) rule_rows(h, nx, ny, dtype, &s);
-        return run_stream(h, in, out, h->scratch, nx, ny, nz, iters, dtype, s, *dev, st);
-    }
+    if (s.kernel == STENCIL_KERNEL_STREAM)
+        return run_stream(h, in, out, h->scratch, nx, ny, nz, iters, dtype, s, *dev, st, rule && plain);
     const void *src = in;
     for (int j = 0; j < iters; ++j) {
         void *dst = ((iters - 1 - j) % 2 == 0) ? out : h->scratch;
@@ -1391,6 +1391,7 @@ struct BatchChain {
     bool tiles = false;
     TilePlan tp;
     stencil_schedule s{};
+    bool rule = false;    // s is the library's rule
     double us = 0;        // estimated time with the device to itself
     int passes = 0;
     int branch = 0;
@@ -1407,14 +1408,13 @@ bool plan_chains(const stencil_batch_item *items, int n, const DevInfo &dev, std
         classes.insert(((b.h->dim * 8 + b.h->r) * 4 + b.dtype) * 2 + b.h->shared);
         BatchChain c;
         c.item = i;
-        const bool rule = chosen_schedule(b.h, b.nx, b.ny, b.nz, b.dtype, &c.s);
+        const bool rule = c.rule = chosen_schedule(b.h, b.nx, b.ny, b.nz, b.dtype, &c.s);
         if (c.s.kernel != STENCIL_KERNEL_STREAM) {
             *rc = STENCIL_ERR_UNSUPPORTED;
             return false;
         }
         if (b.h->checked || b.h->fault_plane >= 0 || b.h->tile_mode < 0) return false;
         c.tiles = rule && plan_tile(b.h, b.nx, b.ny, b.dtype, b.iters, c.s, dev, &c.tp);
-        if (rule && !c.tiles) rule_rows(b.h, b.nx, b.ny, b.dtype, &c.s);
         const int t = c.tiles ? c.tp.t : std::max(1, std::min(c.s.t, b.iters));
         c.passes = (b.iters + t - 1) / t;
         c.us = c.tiles ? c.tp.us
@@ -1484,7 +1484,7 @@ int build_chains(const stencil_batch_item *items, std::vector<BatchChain> &chain
                 rc = run_tiles(b.h, c->tp, b.in, b.out, scr, b.nx, b.ny, b.iters, dev, br[c->branch]);
             else
                 rc = run_stream(b.h, b.in, b.out, scr, b.nx, b.ny, b.nz, b.iters, b.dtype, c->s, dev, br[c->branch],
-                                b.h->dim == 3 ? std::min(1.0, 15.0 * c->us / total) : 1.0);
+                                c->rule, b.h->dim == 3 ? std::min(1.0, 15.0 * c->us / total) : 1.0);
         }
         for (int k = 0; k < nb && err == cudaSuccess; ++k) {
             err = cudaEventRecord(ev[k], br[k]);
@@ -1906,8 +1906,8 @@ int stencil_run_passes(stencil_handle h, int64_t nx, int64_t ny, int64_t nz, int
         return STENCIL_OK;
     }
     if (rag) s = rag_schedule(s, dtype);
-    else if (rule) rule_rows(h, nx, ny, dtype, &s);
     const int t = std::max(1, std::min(s.t, iters));
+    if (rule && !rag) rule_rows(h, nx, ny, dtype, t, &s);
     *out = {rag ? STENCIL_PASS_PADDED : STENCIL_PASS_STREAM, t, (iters + t - 1) / t + (rag ? 1 : 0),
             h->dim == 3 ? s.rows_per_thread : 0, h->dim == 2 ? s.planes_per_step : 0};
     return STENCIL_OK;
@@ -1959,12 +1959,10 @@ int stencil_run_noalloc(stencil_handle h, const void *in, void *out, int64_t nx,
         return run_tiles(h, tp, in, out, nd->scratch, nx, ny, iters, dev, st, pads ? &p : nullptr);
     if (aligned && march_applicable(h, nx, ny, nz, dtype, s))
         return run_march(h, in, out, nd->scratch, nx, ny, nz, iters, dtype, dev, st, pads ? &p : nullptr);
-    if (streamable) {
-        rule_rows(h, nx, ny, dtype, &s);
-        return run_stream(h, in, out, nd->scratch, nx, ny, nz, iters, dtype, s, dev, st);
-    }
+    if (streamable)
+        return run_stream(h, in, out, nd->scratch, nx, ny, nz, iters, dtype, s, dev, st, true);
     if (2 * p.bytes <= kNoAllocScratchBytes && rag_applicable(h, nx, ny, nz, iters, dtype, s))
-        return run_stream(h, in, out, nd->scratch, nx, ny, nz, iters, dtype, rag_schedule(s, dtype), dev, st, 1.0, &p);
+        return run_stream(h, in, out, nd->scratch, nx, ny, nz, iters, dtype, rag_schedule(s, dtype), dev, st, true, 1.0, &p);
     const void *src = in;
     for (int j = 0; j < iters; ++j) {
         void *dst = ((iters - 1 - j) % 2 == 0) ? out : nd->scratch;
