@@ -798,10 +798,12 @@ double stream_run_us(const stencil_plan *h, int64_t nx, int64_t ny, int dtype, i
     static const Fit b16[stn::kMaxR + 1] = {{}, {43, 1.47}, {24, 1.66}, {45, 2.07}, {33, 1.74}, {95, 2.57}, {115, 4.30}};
     static const double shared[stn::kMaxR + 1] = {1, 1, 1.01, 1.05, 1.03, 1, 1};   // one coefficient per distance
     const Fit &f = (dtype == STENCIL_F32 ? f32 : b16)[h->r];
+    // a pass in proportion to its steps; a single step of radius 5 and 6 takes 0.7-0.85 of half a two-step pass
     const int t = std::max(1, std::min(s.t, iters));
+    const double passes = static_cast<double>(iters) / s.t - (h->r >= 5 && iters % s.t == 1 ? 0.25 / s.t : 0.0);
     const int64_t cx = 512 - 2 * round_up((t - 1) * h->r, 4);
     const double mcells = static_cast<double>((nx + cx - 1) / cx * cx) * static_cast<double>(ny) * 1e-6;
-    return (f.fixed + f.per_mcell * mcells) * (h->shared ? shared[h->r] : 1) * iters / s.t;
+    return (f.fixed + f.per_mcell * mcells) * (h->shared ? shared[h->r] : 1) * passes;
 }
 
 // Whether the streaming kernels for rows of any length are compiled for this stencil, at the rows per
@@ -818,7 +820,11 @@ bool rag_compiled(const stencil_plan *h, int dtype, const stencil_schedule &s)
 // without a streaming kernel).  Measured on square FP32 grids (us per step, streaming / tiles):
 // radius 1 at 256^2 12.5 / 0.7, 4096^2 15.6 / 7.7, 16384^2 109 / 98: tiles at every size; radius 2
 // 4096^2 16.5 / 14.6, 8192^2 43 / 53; radius 3 4096^2 23.2 / 20.3, 8192^2 60 / 74; radius 4 4096^2
-// 28.5 / 23.9, 8192^2 70 / 90: the line falls between; radius 6 16384^2 642 / 591.
+// 28.5 / 23.9, 8192^2 70 / 90: the line falls between.  At radius 2 and above tiles are taken from 10 % of
+// estimated gain on: the estimates are good to about that, worst for few steps and for rows of a power of
+// two (one step, streaming / tiles: radius 3 4096^2 27.4 / 31.9, 16384 x 1024 27.5 / 32.0, radius 6 12000^2 279 /
+// 325; 7 steps of radius 4 4096^2 29.8 / 32.0); over 1203 random grids and step counts that leaves none
+// above 1.02 of the streaming passes' time, for 0.2 % of the average gain.
 bool plan_tile(const stencil_plan *h, int64_t nx, int64_t ny, int dtype, int iters, const stencil_schedule &s,
                const DevInfo &dev, TilePlan *tp)
 {
@@ -852,7 +858,8 @@ bool plan_tile(const stencil_plan *h, int64_t nx, int64_t ny, int dtype, int ite
     }
     if (!tp->e) return false;
     if (h->tile_mode > 0) return true;
-    if (s.kernel == STENCIL_KERNEL_STREAM) return tp->us < stream_run_us(h, nx, ny, dtype, iters, s);
+    const double gain = h->r >= 2 ? 0.9 : 1.0;
+    if (s.kernel == STENCIL_KERNEL_STREAM) return tp->us < gain * stream_run_us(h, nx, ny, dtype, iters, s);
     // rows of any length: streaming passes on a padded copy where they are compiled
     return !rag_compiled(h, dtype, s) || tp->us < 2.5 + 1.3e-6 * static_cast<double>(nx) * ny + stream_run_us(h, nx, ny, dtype, iters, s);
 }
