@@ -31,8 +31,11 @@
  *  - The caller owns `in` and `out`; `in` is never written; overlapping `in`
  *    and `out` is rejected (STENCIL_ERR_ALIAS).
  *  - The handle owns a scratch grid (the second buffer of the ping-pong
- *    between passes), allocated with cudaMalloc when a run first needs it
- *    and freed by stencil_destroy.  A handle must not be used from two host
+ *    between passes; two with padded rows where rows are not whole 16-byte
+ *    vectors and the memory can be had), allocated with cudaMalloc when a run
+ *    first needs it and freed by stencil_destroy.  One that a run under
+ *    stream capture has used stays allocated beside a larger one that a later
+ *    run needs (unless that one cannot be had otherwise).  A handle must not be used from two host
  *    threads at once; runs on different streams with the same handle share
  *    the scratch grid and must not overlap on the GPU.
  */

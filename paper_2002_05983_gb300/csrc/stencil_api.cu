@@ -25,6 +25,7 @@
 #include "pack.h"
 #include "pass_rule.h"
 #include "registry.h"
+#include "scratch.h"
 #include "stencil.h"
 #include "sweep_kernel.cuh"
 #include "tile.h"
@@ -36,9 +37,7 @@ struct stencil_plan {
     int checked = 0;             // 1: bounds-checked kernel instantiations (stencil_set_checked)
     int kind() const { return shared + 2 * checked; }   // registry key of the kernel variant
     float c[stn::kMaxK] = {};
-    void *scratch = nullptr;     // second grid of the ping-pong between passes
-    size_t scratch_bytes = 0;
-    int scratch_dev = -1;
+    stn::Scratch scratch;        // second grid of the ping-pong between passes
     void *dev_in = nullptr;      // device copies for stencil_run_host
     void *dev_out = nullptr;
     size_t host_bytes = 0;
@@ -587,38 +586,48 @@ int encode_map(CUtensorMap *m, const void *ptr, int64_t nx, int64_t ny, int64_t 
     return 0;
 }
 
-int ensure_scratch(stencil_plan *h, size_t bytes)
-{
-    int dev = 0;
-    CK(cudaGetDevice(&dev));
-    if (h->scratch && (h->scratch_bytes < bytes || h->scratch_dev != dev)) {
+struct DeviceMemory {
+    const int oom = STENCIL_ERR_OOM;
+    int alloc(void **p, size_t n)
+    {
+        CK(cudaMalloc(p, n));
+        return 0;
+    }
+    int sync()
+    {
         CK(cudaDeviceSynchronize());
-        CK(cudaFree(h->scratch));
-        h->scratch = nullptr;
-        h->scratch_bytes = 0;
+        return 0;
     }
-    if (!h->scratch) {
-        CK(cudaMalloc(&h->scratch, bytes));
-        h->scratch_bytes = bytes;
-        h->scratch_dev = dev;
+    int free(void *p)
+    {
+        CK(cudaFree(p));
+        return 0;
     }
-    return 0;
+};
+
+bool is_capturing(cudaStream_t st)
+{
+    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(st, &cs) != cudaSuccess) (void)cudaGetLastError();   // the launch will tell
+    return cs != cudaStreamCaptureStatusNone;
 }
 
-// As ensure_scratch for a route that another one can stand in for: *ok is false, with no error, where
-// the memory cannot be had (too little of it, or the stream is being captured).
-int try_scratch(stencil_plan *h, size_t bytes, cudaStream_t st, bool *ok)
+// At least `bytes` of scratch for a run.  optional: another route can stand in; *ok is then false, with
+// no error, where the memory cannot be had (too little of it, or the stream is being captured).
+int run_scratch(stencil_plan *h, size_t bytes, bool capturing, bool optional, bool *ok)
 {
     int dev = 0;
     CK(cudaGetDevice(&dev));
-    *ok = h->scratch && h->scratch_bytes >= bytes && h->scratch_dev == dev;
-    if (*ok) return 0;
-    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
-    CK(cudaStreamIsCapturing(st, &cs));
-    if (cs != cudaStreamCaptureStatusNone) return 0;
-    const int rc = ensure_scratch(h, bytes);
-    if (rc && rc != STENCIL_ERR_OOM) return rc;
-    *ok = rc == 0;
+    DeviceMemory m;
+    *ok = h->scratch.fits(bytes, dev);
+    if (!*ok) {
+        const int rc = !optional    ? stn::scratch_need(h->scratch, bytes, dev, m)
+                       : !capturing ? stn::scratch_want(h->scratch, bytes, dev, m, ok)
+                                    : 0;
+        if (rc) return rc;
+        if (!optional) *ok = true;
+    }
+    if (*ok && capturing) h->scratch.captured = true;
     return 0;
 }
 
@@ -1132,52 +1141,54 @@ int run_impl(stencil_plan *h, const void *in, void *out, int64_t nx, int64_t ny,
     if (s.kernel == STENCIL_KERNEL_STREAM && !streamable) return STENCIL_ERR_UNSUPPORTED;
     if (s.kernel == STENCIL_KERNEL_AUTO) s.kernel = streamable ? STENCIL_KERNEL_STREAM : STENCIL_KERNEL_NAIVE;
 
+    const bool cap = is_capturing(st);
     TilePlan tp;
     if (rule && plain && plan_tile(h, nx, ny, dtype, iters, s, *dev, &tp)) {
         bool ok = true;
         if (iters > tp.t && nx % 4) {
             const Padded p = padded(nx, ny, 1, dtype);
-            rc = try_scratch(h, 2 * p.bytes, st, &ok);
+            rc = run_scratch(h, 2 * p.bytes, cap, true, &ok);
             if (rc) return rc;
-            if (ok) return run_tiles(h, tp, in, out, h->scratch, nx, ny, iters, *dev, st, &p);
+            if (ok) return run_tiles(h, tp, in, out, h->scratch.p, nx, ny, iters, *dev, st, &p);
         }
         if (iters > tp.t) {
-            rc = try_scratch(h, bytes, st, &ok);
+            rc = run_scratch(h, bytes, cap, true, &ok);
             if (rc) return rc;
         }
-        if (ok) return run_tiles(h, tp, in, out, h->scratch, nx, ny, iters, *dev, st);
+        if (ok) return run_tiles(h, tp, in, out, h->scratch.p, nx, ny, iters, *dev, st);
     }
 
     if (rule && plain && march_applicable(h, nx, ny, nz, dtype, s)) {
         const Padded p = padded(nx, ny, nz, dtype);
         bool ok = true, pads = nx % 4 != 0 && iters > 1;
         if (pads) {
-            rc = try_scratch(h, 2 * p.bytes, st, &pads);
+            rc = run_scratch(h, 2 * p.bytes, cap, true, &pads);
             if (rc) return rc;
         }
         if (iters > 1 && !pads) {
-            rc = try_scratch(h, bytes, st, &ok);
+            rc = run_scratch(h, bytes, cap, true, &ok);
             if (rc) return rc;
         }
-        if (ok) return run_march(h, in, out, h->scratch, nx, ny, nz, iters, dtype, *dev, st, pads ? &p : nullptr);
+        if (ok) return run_march(h, in, out, h->scratch.p, nx, ny, nz, iters, dtype, *dev, st, pads ? &p : nullptr);
     }
     if (rule && plain && rag_applicable(h, nx, ny, nz, iters, dtype, s)) {
         const Padded p = padded(nx, ny, nz, dtype);
         bool ok = true;
-        rc = try_scratch(h, 2 * p.bytes, st, &ok);
+        rc = run_scratch(h, 2 * p.bytes, cap, true, &ok);
         if (rc) return rc;
-        if (ok) return run_stream(h, in, out, h->scratch, nx, ny, nz, iters, dtype, rag_schedule(s, dtype), *dev, st, true, 1.0, &p);
+        if (ok) return run_stream(h, in, out, h->scratch.p, nx, ny, nz, iters, dtype, rag_schedule(s, dtype), *dev, st, true, 1.0, &p);
     }
     const int t = s.kernel == STENCIL_KERNEL_NAIVE ? 1 : std::max(1, std::min(s.t, iters));
     if (iters > t) {
-        rc = ensure_scratch(h, bytes);
+        bool ok = true;
+        rc = run_scratch(h, bytes, cap, false, &ok);
         if (rc) return rc;
     }
     if (s.kernel == STENCIL_KERNEL_STREAM)
-        return run_stream(h, in, out, h->scratch, nx, ny, nz, iters, dtype, s, *dev, st, rule && plain);
+        return run_stream(h, in, out, h->scratch.p, nx, ny, nz, iters, dtype, s, *dev, st, rule && plain);
     const void *src = in;
     for (int j = 0; j < iters; ++j) {
-        void *dst = ((iters - 1 - j) % 2 == 0) ? out : h->scratch;
+        void *dst = ((iters - 1 - j) % 2 == 0) ? out : h->scratch.p;
         rc = launch_naive(h, src, dst, nx, ny, nz, dtype, st, *dev);
         if (rc) return rc;
         src = dst;
@@ -1781,9 +1792,11 @@ int stencil_destroy(stencil_handle h)
 {
     if (!h) return STENCIL_OK;
     int rc = STENCIL_OK;
-    if (h->scratch || h->dev_in || h->dev_out) {
+    if (h->scratch.p || h->scratch.kept || h->dev_in || h->dev_out) {
         if (cudaDeviceSynchronize() != cudaSuccess) rc = STENCIL_ERR_CUDA;
-        if (h->scratch) cudaFree(h->scratch);
+        DeviceMemory m;
+        stn::scratch_free_kept(h->scratch, m);
+        if (h->scratch.p) cudaFree(h->scratch.p);
         if (h->dev_in) cudaFree(h->dev_in);
         if (h->dev_out) cudaFree(h->dev_out);
     }
