@@ -1151,10 +1151,13 @@ int run_impl(stencil_plan *h, const void *in, void *out, int64_t nx, int64_t ny,
             if (rc) return rc;
             if (ok) return run_tiles(h, tp, in, out, h->scratch.p, nx, ny, iters, *dev, st, &p);
         }
-        if (iters > tp.t) {
+        // A single pass needs none, but a longer run of the same problem may come under stream capture, which
+        // cannot allocate: what the schedule's own passes would need is there after any warm-up.
+        if (iters > tp.t || iters > (s.kernel == STENCIL_KERNEL_NAIVE ? 1 : s.t)) {
             rc = run_scratch(h, bytes, cap, true, &ok);
             if (rc) return rc;
         }
+        if (iters <= tp.t) ok = true;
         if (ok) return run_tiles(h, tp, in, out, h->scratch.p, nx, ny, iters, *dev, st);
     }
 
