@@ -2064,6 +2064,7 @@ int stencil_resolve_schedule(stencil_handle h, int64_t nx, int64_t ny, int64_t n
     chosen_schedule(h, nx, ny, nz, dtype, &s);
     if (sched) {
         if (sched->t) s.t = sched->t;
+        if (h->dim == 3 && sched->t) s.rows_per_thread = 2;   // as stencil_run_ex
         if (sched->rows_per_thread) s.rows_per_thread = sched->rows_per_thread;
         if (sched->seg) s.seg = sched->seg;
         if (sched->threads_x) s.threads_x = sched->threads_x;
@@ -2088,6 +2089,7 @@ int stencil_schedule_features(stencil_handle h, int64_t nx, int64_t ny, int64_t 
     default_schedule(h, nx, ny, nz, dtype, &s);
     if (sched) {
         if (sched->t) s.t = sched->t;
+        if (h->dim == 3 && sched->t) s.rows_per_thread = 2;   // as stencil_run_ex
         if (sched->rows_per_thread) s.rows_per_thread = sched->rows_per_thread;
         if (sched->seg) s.seg = sched->seg;
         if (sched->threads_x) s.threads_x = sched->threads_x;
