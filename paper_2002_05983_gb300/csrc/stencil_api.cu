@@ -1978,9 +1978,11 @@ int stencil_run_noalloc(stencil_handle h, const void *in, void *out, int64_t nx,
     TilePlan tp;
     const Padded p = padded(nx, ny, nz, dtype);
     const bool pads = nx % 4 && 2 * p.bytes <= kNoAllocScratchBytes;   // two padded grids fit
-    if (aligned && plan_tile(h, nx, ny, dtype, iters, s, dev, &tp))
+    // rows that are not whole vectors run from any address, like in stencil_run
+    const bool any = aligned || s.kernel == STENCIL_KERNEL_NAIVE;
+    if (any && plan_tile(h, nx, ny, dtype, iters, s, dev, &tp))
         return run_tiles(h, tp, in, out, nd->scratch, nx, ny, iters, dev, st, pads ? &p : nullptr);
-    if (aligned && march_applicable(h, nx, ny, nz, dtype, s))
+    if (any && march_applicable(h, nx, ny, nz, dtype, s))
         return run_march(h, in, out, nd->scratch, nx, ny, nz, iters, dtype, dev, st, pads ? &p : nullptr);
     if (streamable)
         return run_stream(h, in, out, nd->scratch, nx, ny, nz, iters, dtype, s, dev, st, true);
