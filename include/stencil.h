@@ -375,7 +375,11 @@ int stencil_run_passes(stencil_handle h, int64_t nx, int64_t ny, int64_t nz, int
  * status (read with stencil_get_device_status).  Only a few configurations
  * are compiled checked (2D FP32 r=1 t=1,5, r=4 t=2, r=6 t=2; 2D BF16 r=2
  * t=3; 3D FP32 r=1 t=2 2 rows, r=3 t=1 4 rows, r=5 t=1 2 rows; 3D FP16 r=2
- * t=1 2 rows); other schedules return UNSUPPORTED.  on = 0 restores the
+ * t=1 2 rows); other schedules return UNSUPPORTED.  Where stencil_set_tile asks
+ * for them (modes 1 to 3), the rule's other kernels run checked too: register
+ * tiles FP32 r=1 (4 rows per thread), r=3, r=6 (8), shared r=2 (16), BF16 r=4
+ * (16); marching passes FP32 r=1, 4, shared r=2, FP16 r=3; rows of any length in
+ * 3D FP32 r=1, 4 and FP16 r=2, and 2D FP32 r=4.  on = 0 restores the
  * normal kernels.  Errors: INVALID_ARG. */
 int stencil_set_checked(stencil_handle h, int on);
 

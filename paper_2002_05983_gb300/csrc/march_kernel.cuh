@@ -7,7 +7,7 @@
 // loaded r planes earlier: L1 hits.  Nothing is staged in shared memory and no step has a barrier, so a
 // run of one to four planes costs no pipeline fill and a 64 x 16 tile gives a block per few planes:
 // what a small grid needs to fill 152 SMs.  Bound by latency there (0.4 us a plane for a lone block;
-// 64^3 radius 2: 2.9 us a pass, the streaming kernel 4.5; 96^3 radius 4: 5.4 against 9.3), and by L1
+// 64^3 radius 2: 2.8 us a pass, the streaming kernel 4.0; 96^3 radius 4: 5.4 against 9.3), and by L1
 // throughput where there are many planes per SM (2r+1 vector loads a cell vector; 256^3 radius 2: 37
 // us, streaming 25).  Two rows per thread measured slower at every size (130-180 registers).
 #pragma once
@@ -27,10 +27,13 @@ struct MarchArgs {
     int ntx, nty;           // tiles in x and y
     int vout;               // 4-cell vector stores
     float c[kMaxK];
+    unsigned *status;       // bounds-checked kernels: device status word
 };
 
-// V: vector loads (rows start on whole 4-cell vectors); else cell by cell.
-template <int R, typename S, bool SH, bool V>
+// V: vector loads (rows start on whole 4-cell vectors); else cell by cell.  CHK: every load must lie in the input's
+// rows (to the pitch's end with vectors) and every store in the output's; one that does not sets kStatusBounds
+// and is skipped.
+template <int R, typename S, bool SH, bool V, bool CHK = false>
 __global__ void __launch_bounds__(kMarchThreads) march3d_kernel(const __grid_constant__ MarchArgs a)
 {
     static_assert(R <= 4, "one vector of x neighbours per side");
@@ -60,7 +63,19 @@ __global__ void __launch_bounds__(kMarchThreads) march3d_kernel(const __grid_con
         offd[m] = min(gy0 + VY + m, a.ny - 1) * a.pin + gxc;
     }
     const S *in = static_cast<const S *>(a.in);
+    auto ok = [&](int64_t at, int n, int64_t limit) -> bool {
+        if constexpr (CHK) {
+            if (at >= 0 && at + n <= limit) return true;
+            atomicOr(a.status, kStatusBounds);
+            return false;
+        } else {
+            return true;
+        }
+    };
+    // the last row ends with its cells, or with the pitch where vectors reach over them
+    auto ok_in = [&](const S *p, int n) { return ok(p - in, n, plane * a.nz - (V ? 0 : a.pin - a.nx)); };
     auto load = [&](const S *p, float (&v)[4]) {   // p: cell gxc of a row
+        if (!ok_in(p, V ? 4 : 1 + min(3, a.nx - 1 - gxc))) return;
         if constexpr (V) {
             Fmt<S>::load4(p, v);
         } else {
@@ -117,7 +132,8 @@ __global__ void __launch_bounds__(kMarchThreads) march3d_kernel(const __grid_con
                         load(pc + off[v] - 4, t);
                     } else {
 #pragma unroll
-                        for (int c = 0; c < 4; ++c) t[c] = cell_in<S>(pc + off[v] - 4 + c);
+                        for (int c = 0; c < 4; ++c)
+                            if (ok_in(pc + off[v] - 4 + c, 1)) t[c] = cell_in<S>(pc + off[v] - 4 + c);
                     }
 #pragma unroll
                     for (int k = 0; k < R; ++k) xl[k] = t[3 - k];
@@ -132,7 +148,8 @@ __global__ void __launch_bounds__(kMarchThreads) march3d_kernel(const __grid_con
                         for (int c = 1; c < 4; ++c) t[c] = 4 + c > cr ? t[c - 1] : t[c];
                     } else {
 #pragma unroll
-                        for (int c = 0; c < 4; ++c) t[c] = cell_in<S>(pc + off[v] + min(4 + c, cr));
+                        for (int c = 0; c < 4; ++c)
+                            if (ok_in(pc + off[v] + min(4 + c, cr), 1)) t[c] = cell_in<S>(pc + off[v] + min(4 + c, cr));
                     }
 #pragma unroll
                     for (int k = 0; k < R; ++k) xr[k] = t[k];
@@ -177,6 +194,7 @@ __global__ void __launch_bounds__(kMarchThreads) march3d_kernel(const __grid_con
                 }
                 if (gx < a.nx && gy0 + v < a.ny) {
                     S *o = out + (static_cast<int64_t>(z) * a.ny + gy0 + v) * a.pout + gx;
+                    if (!ok(o - out, a.vout ? 4 : min(4, a.nx - gx), static_cast<int64_t>(a.pout) * a.ny * a.nz)) continue;
                     if (a.vout) {
                         Fmt<S>::store4(o, res);
                     } else {

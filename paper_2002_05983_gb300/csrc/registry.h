@@ -69,6 +69,7 @@ int list_rag_f32_wide(const KernelEntry **e);
 int list_rag_bf16(const KernelEntry **e);
 int list_rag_f16(const KernelEntry **e);
 int list_rag_2d(const KernelEntry **e);
+int list_rag_checked(const KernelEntry **e);
 
 }  // namespace stn
 
@@ -82,10 +83,11 @@ int list_rag_2d(const KernelEntry **e);
      reinterpret_cast<const void *>(&stn::sweep_kernel<D, R, T, VY, S, TX, TY, SH, CHK, P>),         \
      reinterpret_cast<const void *>(&stn::sweep_persistent<D, R, T, VY, S, TX, TY, SH, CHK, P>))
 // rows of any length (kind + 4): no persistent form
-#define STN_ER(D, R, T, VY, S, DT, SH, P)                                                          \
-    STN_ANY(D, R, T, VY, S, DT, (D == 2 ? 128 : 16), (D == 2 ? 1 : 8), P, (SH ? 1 : 0) + 4,             \
+#define STN_ER(D, R, T, VY, S, DT, SH, P) STN_ERC(D, R, T, VY, S, DT, SH, false, P)
+#define STN_ERC(D, R, T, VY, S, DT, SH, CHK, P)                                                    \
+    STN_ANY(D, R, T, VY, S, DT, (D == 2 ? 128 : 16), (D == 2 ? 1 : 8), P, (SH ? 1 : 0) + (CHK ? 2 : 0) + 4,   \
      reinterpret_cast<const void *>(                                                              \
-         &stn::sweep_kernel<D, R, T, VY, S, (D == 2 ? 128 : 16), (D == 2 ? 1 : 8), SH, false, P, true>),  \
+         &stn::sweep_kernel<D, R, T, VY, S, (D == 2 ? 128 : 16), (D == 2 ? 1 : 8), SH, CHK, P, true>),    \
      nullptr)
 #define STN_ANY(D, R, T, VY, S, DT, TX, TY, P, KIND, FN, PFN)                                         \
     {D, R, T, VY, DT, KIND, TX, TY, P, STN_G(D, R, T, VY, S, TX, TY, P)::QP,  \

@@ -104,7 +104,7 @@ struct Registry {
                            stn::list_2d_f32sh,   stn::list_3d_f32sh,   stn::list_checked,  stn::list_2d_f32_p2,
                            stn::list_2d_bf16_p2, stn::list_2d_f16_p2,  stn::list_2d_p4,      stn::list_2d_p2_wide,
                            stn::list_rag_f32,    stn::list_rag_f32_wide, stn::list_rag_bf16,  stn::list_rag_f16,
-                           stn::list_rag_2d};
+                           stn::list_rag_2d,     stn::list_rag_checked};
         for (L f : lists) {
             const stn::KernelEntry *e = nullptr;
             const int n = f(&e);
@@ -709,7 +709,7 @@ const std::vector<stn::TileEntry> &tile_entries()
     static const std::vector<stn::TileEntry> all = [] {
         std::vector<stn::TileEntry> v;
         for (auto f : {stn::list_tile_r1, stn::list_tile_r2, stn::list_tile_r3, stn::list_tile_r4, stn::list_tile_r5,
-                       stn::list_tile_r6}) {
+                       stn::list_tile_r6, stn::list_tile_checked}) {
             const stn::TileEntry *e = nullptr;
             const int n = f(&e);
             v.insert(v.end(), e, e + n);
@@ -718,6 +718,9 @@ const std::vector<stn::TileEntry> &tile_entries()
     }();
     return all;
 }
+
+// A checked handle takes the rule's other kernels only where stencil_set_tile asks for them.
+bool checked_ok(const stencil_plan *h) { return !h->checked || h->tile_mode > 0; }
 
 struct TileGrid {
     int h, hx, ntx, nty;
@@ -739,7 +742,7 @@ bool tile_grid(const stn::TileEntry &e, int64_t nx, int64_t ny, int t, TileGrid 
 }
 
 int tile_launch(const stencil_plan *h, const stn::TileEntry &e, int t, int rnd, const void *in, void *out, int64_t nx,
-                int64_t ny, int64_t pin, int64_t pout, cudaStream_t st)
+                int64_t ny, int64_t pin, int64_t pout, const DevInfo &dev, cudaStream_t st)
 {
     TileGrid g;
     if (!tile_grid(e, nx, ny, t, &g)) return STENCIL_ERR_UNSUPPORTED;
@@ -759,6 +762,7 @@ int tile_launch(const stencil_plan *h, const stn::TileEntry &e, int t, int rnd, 
     a.vin = pin % 4 == 0 && reinterpret_cast<uintptr_t>(in) % vec == 0;
     a.vout = pout % 4 == 0 && reinterpret_cast<uintptr_t>(out) % vec == 0;
     std::memcpy(a.c, h->c, sizeof(float) * h->K);
+    a.status = dev.status;
     void *args[] = {&a};
     return launch_pass(e.fn, dim3(static_cast<unsigned>(g.ntx) * static_cast<unsigned>(g.nty)),
                        dim3(static_cast<unsigned>(32 * e.w)), args, e.smem, st, true);
@@ -837,12 +841,12 @@ bool rag_compiled(const stencil_plan *h, int dtype, const stencil_schedule &s)
 bool plan_tile(const stencil_plan *h, int64_t nx, int64_t ny, int dtype, int iters, const stencil_schedule &s,
                const DevInfo &dev, TilePlan *tp)
 {
-    if (h->dim != 2 || h->checked || h->fault_plane >= 0 || h->tile_mode < 0 || h->tile_mode == 2) return false;
+    if (h->dim != 2 || h->fault_plane >= 0 || h->tile_mode < 0 || h->tile_mode == 2 || !checked_ok(h)) return false;
     if (nx > (1 << 30) || ny > (1 << 30)) return false;   // coordinates past the grid stay ints
     tp->rnd = s.kernel == STENCIL_KERNEL_STREAM && dtype != STENCIL_F32 ? s.t : 1;
     tp->e = nullptr;
     for (const auto &e : tile_entries()) {
-        if (e.r != h->r || e.dtype != dtype || e.sh != h->shared || e.smem > static_cast<size_t>(dev.max_smem)) continue;
+        if (e.r != h->r || e.dtype != dtype || e.sh != h->shared || e.chk != h->checked || e.smem > static_cast<size_t>(dev.max_smem)) continue;
         if (h->tile_v && e.v != h->tile_v) continue;
         int prev = 0;
         for (int t = 1; t <= std::min(iters, 32); ++t) {
@@ -904,7 +908,7 @@ int run_tiles(const stencil_plan *h, const TilePlan &tp, const void *in, void *o
         void *dst = rag ? (j == L - 1 ? out : static_cast<char *>(scratch) + (j & 1) * rag->bytes)
                         : ((L - 1 - j) % 2 == 0) ? out : scratch;
         const int64_t pout = rag && j < L - 1 ? rag->pitch : nx;
-        rc = tile_launch(h, *tp.e, tile_steps(iters, L, unit, j), unit, src, dst, nx, ny, pin, pout, st);
+        rc = tile_launch(h, *tp.e, tile_steps(iters, L, unit, j), unit, src, dst, nx, ny, pin, pout, dev, st);
         if (rc) return rc;
         src = dst;
         pin = pout;
@@ -1002,7 +1006,8 @@ const stn::MarchEntry *march_entry(const stencil_plan *h, int dtype, bool vec)
 {
     static const std::vector<stn::MarchEntry> all = [] {
         std::vector<stn::MarchEntry> v;
-        for (auto f : {stn::list_march_r1, stn::list_march_r2, stn::list_march_r3, stn::list_march_r4}) {
+        for (auto f : {stn::list_march_r1, stn::list_march_r2, stn::list_march_r3, stn::list_march_r4,
+                       stn::list_march_checked}) {
             const stn::MarchEntry *e = nullptr;
             const int n = f(&e);
             v.insert(v.end(), e, e + n);
@@ -1010,7 +1015,7 @@ const stn::MarchEntry *march_entry(const stencil_plan *h, int dtype, bool vec)
         return v;
     }();
     for (const auto &e : all)
-        if (e.r == h->r && e.dtype == dtype && e.sh == h->shared && e.vec == (vec ? 1 : 0)) return &e;
+        if (e.r == h->r && e.dtype == dtype && e.sh == h->shared && e.vec == (vec ? 1 : 0) && e.chk == h->checked) return &e;
     return nullptr;
 }
 
@@ -1042,6 +1047,7 @@ int run_march(const stencil_plan *h, const void *in, void *out, void *scratch, i
                                                 static_cast<int64_t>(dev.sms) * std::max(fi.occ, 1), 2 * h->r));
         a.vout = pout % 4 == 0 && reinterpret_cast<uintptr_t>(dst) % vec == 0;
         std::memcpy(a.c, h->c, sizeof(float) * h->K);
+        a.status = dev.status;
         const int64_t blocks = static_cast<int64_t>(a.ntx) * a.nty * ((nz + a.seg - 1) / a.seg);
         if (blocks > 0x7fffffffLL) return STENCIL_ERR_UNSUPPORTED;
         void *args[] = {&a};
@@ -1070,7 +1076,7 @@ double naive_step_us(const stencil_plan *h, double mcells)
 // steps, is within 9 % either way between 64^3 and 128^3.
 bool march_applicable(const stencil_plan *h, int64_t nx, int64_t ny, int64_t nz, int dtype, const stencil_schedule &s)
 {
-    if (h->dim != 3 || h->checked || h->fault_plane >= 0 || h->tile_mode < 0 || h->tile_mode == 2) return false;
+    if (h->dim != 3 || h->fault_plane >= 0 || h->tile_mode < 0 || h->tile_mode == 2 || !checked_ok(h)) return false;
     const bool stream = s.kernel == STENCIL_KERNEL_STREAM;
     if (!march_entry(h, dtype, true) || (dtype != STENCIL_F32 && stream && s.t != 1)) return false;
     if (nx > (1 << 30) || (nx + 8) * ny > (1LL << 30) || nz > (1 << 23)) return false;   // offsets within a plane stay ints
@@ -1093,7 +1099,7 @@ stencil_schedule rag_schedule(stencil_schedule s, int dtype)
 // copy and the passes are estimated below the one-step kernel's time.
 bool rag_applicable(const stencil_plan *h, int64_t nx, int64_t ny, int64_t nz, int iters, int dtype, const stencil_schedule &s0)
 {
-    if (s0.kernel != STENCIL_KERNEL_NAIVE || h->checked || h->fault_plane >= 0 || h->tile_mode < 0) return false;
+    if (s0.kernel != STENCIL_KERNEL_NAIVE || h->fault_plane >= 0 || h->tile_mode < 0 || !checked_ok(h)) return false;
     if (nx > (1 << 30) || ny > (1 << 30) || nz > (1 << 30)) return false;   // coordinates past the grid stay ints
     const stencil_schedule s = rag_schedule(s0, dtype);
     if (!rag_compiled(h, dtype, s)) return false;

@@ -73,9 +73,11 @@ template <int D, int R, int T, int VY, int ES, int TX, int TY, int P = 1> struct
     static constexpr int BODY = T * VY * 4 * (2 * D * R + 1);
     static constexpr bool ROT = D == 2 || QP * BODY <= kRotMaxFma;
     // 3D one-level kernels of radius 4 to 6, and of radius 2 with 16-bit storage and 4 rows per
-    // thread, take two steps per chunk: half the moves for VY * 8 more registers, which cost them no
-    // resident block (512^3, one step / two: FP32 radius 4 217.9 / 212.5 us a pass, 5 330 / 302, 6 412
-    // / 380; 16-bit radius 2 140.8 / 131.4, 4 262 / 236; FP32 radius 3 loses one: 170 / 221).
+    // thread, take two steps per chunk: half the moves for VY * 8 more registers and, where the ring
+    // rounds up to whole chunks, one more plane in it (512^3, one step / two: FP32 radius 4 217.9 / 212.5 us
+    // a pass, 5 330 / 302, 6 412 / 380; 16-bit radius 2 140.8 / 131.4, 4 262 / 236).  No resident block is lost
+    // but by FP32 radius 4 with 2 rows, 4 -> 3 for the larger ring: 0.83-0.98 of the time all the same, 1.10
+    // where four blocks per SM held a whole grid (704 x 700 x 64).  FP32 radius 3 loses one: 170 / 221.
     static constexpr bool TWO = D == 3 && T == 1 && (R >= 4 || (R == 2 && VY == 4 && ES == 2));
     static constexpr int U = ROT ? QP / P : TWO ? 2 : (kChunkFma / BODY >= 1 ? kChunkFma / BODY : 1);
     static constexpr int NQ = ROT ? QP : QP + U;       // queue registers per level and cell

@@ -181,8 +181,8 @@ __device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c)
 // it): the next pass's blocks may take their places as soon as every block of this one has
 // started, and set themselves up; they read and write grids only after grid_dep_wait, which
 // returns when all work before this launch is complete (at once in any other launch).  3D passes
-// use it (512^3, radius 1..4: 1 % faster; 96^3, one-wave blocks: 6.8 -> 5.9 us per pass); 2D
-// streaming passes don't: blocks placed as slots come free lose the order in which neighbouring
+// use it where they fill the device (pass_rule.h; 512^3, radius 1..4: 1 % faster; 96^3, one-wave blocks:
+// 6.8 -> 5.9 us per pass); 2D streaming passes don't: blocks placed as slots come free lose the order in which neighbouring
 // strips share L2 (16384^2 radius 4 0.4 %, 8192^2 2.6 % slower with it).
 __device__ __forceinline__ void grid_dep_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void grid_dep_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
@@ -707,10 +707,11 @@ __device__ __forceinline__ bool sweep_tile(const CUtensorMap *tmap, const SweepA
             uint32_t bytes = xb > xa ? static_cast<uint32_t>((xb - xa) * sizeof(S)) : 0u;
             const int nq = P == 1 ? 1 : min(P, lmax - P * kq + 1);   // planes of this step inside the grid
             if constexpr (CHK) {   // destination inside the slot, source inside the grid, 16-byte units
-                const int64_t src = static_cast<int64_t>(P * kq) * a.nx + xa;
+                const int pin = RAG ? a.pin : a.nx;
+                const int64_t src = static_cast<int64_t>(P * kq) * pin + xa;
                 const bool ok = xa - ox_in >= 0 && (xa - ox_in) * sizeof(S) + bytes <= SLOTIN * sizeof(S) &&
-                                src >= 0 && (src + static_cast<int64_t>(nq - 1) * a.nx) * sizeof(S) + bytes <=
-                                                static_cast<int64_t>(a.nx) * a.ns * sizeof(S) &&
+                                src >= 0 && (src + static_cast<int64_t>(nq - 1) * pin) * sizeof(S) + bytes <=
+                                                static_cast<int64_t>(pin) * a.ns * sizeof(S) &&
                                 bytes % 16 == 0 && (src * sizeof(S)) % 16 == 0 && ((xa - ox_in) * sizeof(S)) % 16 == 0;
                 if (!ok) {
                     atomicOr(a.status, kStatusBounds);
@@ -996,9 +997,10 @@ __device__ __forceinline__ bool sweep_tile(const CUtensorMap *tmap, const SweepA
                 for (int vy = 0; vy < VY; ++vy)
                     if (ystore[vy]) {
                         if constexpr (CHK) {   // inside the output grid, four whole cells of one row
-                            const int64_t e = (o + vy * a.nx) - static_cast<S *>(a.out);
-                            const int64_t total = static_cast<int64_t>(a.nx) * a.ny * a.nz;
-                            if (e < 0 || e + 4 > total || gx + 4 > a.nx) {
+                            const int64_t e = (o + static_cast<int64_t>(vy) * pout) - static_cast<S *>(a.out);
+                            const int64_t total = static_cast<int64_t>(pout) * a.ny * a.nz;
+                            const int n = RAG && a.dense ? min(4, a.nxr - gx) : 4;   // cells stored
+                            if (e < 0 || n < 1 || e + n > total || gx + n > (RAG && a.dense ? a.nxr : a.nx)) {
                                 atomicOr(a.status, kStatusBounds);
                                 continue;
                             }

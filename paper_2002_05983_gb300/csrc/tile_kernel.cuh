@@ -58,6 +58,7 @@ struct TileArgs {
     int ntx;              // tiles per tile row
     int vin, vout;        // rows start on whole 4-cell vectors: vector loads / stores
     float c[kMaxK2];
+    unsigned *status;     // bounds-checked kernels: device status word
 };
 
 template <int R, int V, int W> struct TileGeo {
@@ -92,8 +93,9 @@ template <> __device__ __forceinline__ float cell_in<__half>(const __half *p) { 
 __device__ __forceinline__ float4 f4(const float (&v)[4]) { return make_float4(v[0], v[1], v[2], v[3]); }
 __device__ __forceinline__ void set4(float (&v)[4], float4 t) { v[0] = t.x; v[1] = t.y; v[2] = t.z; v[3] = t.w; }
 
-// Tile `blk` of one pass.
-template <int R, int V, int W, typename S, bool SH, typename A>
+// Tile `blk` of one pass.  CHK: every global load and store must lie in the rows' cells and every shared-memory
+// access in the exchange buffer; one that does not sets kStatusBounds and is skipped.
+template <int R, int V, int W, typename S, bool SH, bool CHK, typename A>
 __device__ __forceinline__ void tile2d(const A &a, int blk, float4 *halo)
 {
     using G = TileGeo<R, V, W>;
@@ -107,21 +109,38 @@ __device__ __forceinline__ void tile2d(const A &a, int blk, float4 *halo)
     const bool xedge = ox < 0 || ox + kTileW > a.nx;
     const bool last_y = oy + TH >= a.ny;
 
+    auto ok = [&](int64_t at, int n, int64_t limit) -> bool {
+        if constexpr (CHK) {
+            if (at >= 0 && at + n <= limit) return true;
+            atomicOr(a.status, kStatusBounds);
+            return false;
+        } else {
+            return true;
+        }
+    };
+    auto ok_in = [&](int64_t at, int n) { return ok(at, n, static_cast<int64_t>(a.ny - 1) * a.pin + a.nx); };
+    auto ok_out = [&](int64_t at, int n) { return ok(at, n, static_cast<int64_t>(a.ny - 1) * a.pout + a.nx); };
+    auto ok_halo = [&](const float4 *p) { return ok(p - halo, 1, 2 * W * NB * 32); };
+
     float q[V][4];
     if (live) {
         const S *in = static_cast<const S *>(a.in);
         if (a.vin && gx >= 0 && gx + 4 <= a.nx) {
 #pragma unroll
-            for (int v = 0; v < V; ++v) Fmt<S>::load4(in + static_cast<int64_t>(min(gy0 + v, a.ny - 1)) * a.pin + gx, q[v]);
+            for (int v = 0; v < V; ++v) {
+                const int64_t at = static_cast<int64_t>(min(gy0 + v, a.ny - 1)) * a.pin + gx;
+                if (ok_in(at, 4)) Fmt<S>::load4(in + at, q[v]);
+            }
         } else {
             int xc[4];
 #pragma unroll
             for (int c = 0; c < 4; ++c) xc[c] = min(max(gx + c, 0), a.nx - 1);
 #pragma unroll
             for (int v = 0; v < V; ++v) {
-                const S *row = in + static_cast<int64_t>(min(gy0 + v, a.ny - 1)) * a.pin;
+                const int64_t row = static_cast<int64_t>(min(gy0 + v, a.ny - 1)) * a.pin;
 #pragma unroll
-                for (int c = 0; c < 4; ++c) q[v][c] = cell_in<S>(row + xc[c]);
+                for (int c = 0; c < 4; ++c)
+                    if (ok_in(row + xc[c], 1)) q[v][c] = cell_in<S>(in + row + xc[c]);
             }
         }
     }
@@ -162,7 +181,8 @@ __device__ __forceinline__ void tile2d(const A &a, int blk, float4 *halo)
         float4 *buf = halo + (s & 1) * (W * NB * 32) + lane;
         if (live) {
 #pragma unroll
-            for (int k = 0; k < NB; ++k) buf[(w * NB + k) * 32] = f4(q[(NB < 2 * R || k < R) ? k : V - 2 * R + k]);
+            for (int k = 0; k < NB; ++k)
+                if (ok_halo(buf + (w * NB + k) * 32)) buf[(w * NB + k) * 32] = f4(q[(NB < 2 * R || k < R) ? k : V - 2 * R + k]);
         }
         __syncthreads();
         ++s;
@@ -173,9 +193,9 @@ __device__ __forceinline__ void tile2d(const A &a, int blk, float4 *halo)
             float up[R][4], dn[R][4];
 #pragma unroll
             for (int m = 0; m < R; ++m) {
-                if (w > 0) set4(up[m], buf[((w - 1) * NB + NB - 1 - m) * 32]);
+                if (w > 0 && ok_halo(buf + ((w - 1) * NB + NB - 1 - m) * 32)) set4(up[m], buf[((w - 1) * NB + NB - 1 - m) * 32]);
                 else set4(up[m], f4(q[0]));
-                if (!below && w < W - 1) set4(dn[m], buf[((w + 1) * NB + m) * 32]);
+                if (!below && w < W - 1 && ok_halo(buf + ((w + 1) * NB + m) * 32)) set4(dn[m], buf[((w + 1) * NB + m) * 32]);
                 else set4(dn[m], f4(q[V - 1]));
             }
             auto yn = [&](int y) -> const float * {   // row y of the old field, -R <= y < V + R
@@ -261,7 +281,8 @@ __device__ __forceinline__ void tile2d(const A &a, int blk, float4 *halo)
 #pragma unroll
                 for (int v = 0; v < V; ++v) {
                     const int y = w * V + v;
-                    if (y >= r0 && y < r1 && gy0 + v < a.ny) Fmt<S>::store4(out + static_cast<int64_t>(v) * a.pout, q[v]);
+                    if (y >= r0 && y < r1 && gy0 + v < a.ny && ok_out(static_cast<int64_t>(gy0 + v) * a.pout + gx, 4))
+                        Fmt<S>::store4(out + static_cast<int64_t>(v) * a.pout, q[v]);
                 }
             } else {
 #pragma unroll
@@ -270,7 +291,8 @@ __device__ __forceinline__ void tile2d(const A &a, int blk, float4 *halo)
                     if (y >= r0 && y < r1 && gy0 + v < a.ny) {
 #pragma unroll
                         for (int c = 0; c < 4; ++c)
-                            if (gx + c < a.nx) out[static_cast<int64_t>(v) * a.pout + c] = to_storage<S>(q[v][c]);
+                            if (gx + c < a.nx && ok_out(static_cast<int64_t>(gy0 + v) * a.pout + gx + c, 1))
+                                out[static_cast<int64_t>(v) * a.pout + c] = to_storage<S>(q[v][c]);
                     }
                 }
             }
@@ -279,13 +301,13 @@ __device__ __forceinline__ void tile2d(const A &a, int blk, float4 *halo)
 }
 
 // One pass over the grid, one tile per block.
-template <int R, int V, int W, typename S, bool SH>
+template <int R, int V, int W, typename S, bool SH, bool CHK = false>
 __global__ void __launch_bounds__(32 * W, V <= 8 ? 2 : 1) tile2d_kernel(const __grid_constant__ TileArgs a)
 {
     extern __shared__ __align__(1024) unsigned char smem[];
     grid_dep_launch();
     grid_dep_wait();
-    tile2d<R, V, W, S, SH>(a, static_cast<int>(blockIdx.x), reinterpret_cast<float4 *>(smem));
+    tile2d<R, V, W, S, SH, CHK>(a, static_cast<int>(blockIdx.x), reinterpret_cast<float4 *>(smem));
 }
 
 }  // namespace stn
