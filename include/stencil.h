@@ -141,7 +141,9 @@ int stencil_create(stencil_handle *out, int dim, int radius, const float *coeffs
  * the 2*dim neighbours at distance i (clamped as above) summed left to right
  * in FP32, then one FMA per distance (FP32 path: one rounded multiply, then per
  * distance 2*dim-1 rounded adds and one FMA).  Streaming kernels exist for FP32
- * storage, radius 1..4; other cases run the one-step-per-launch kernel.
+ * storage, radius 1..4, register tiles (2D) for FP32 storage and every radius,
+ * marching passes (3D) for FP32 and radius 1..4; other cases run the
+ * one-step-per-launch kernel.
  * Errors: INVALID_ARG. */
 int stencil_create_shared(stencil_handle *out, int dim, int radius, const float *coeffs);
 
@@ -211,6 +213,12 @@ int stencil_default_schedule(stencil_handle h, int64_t nx, int64_t ny, int64_t n
  *    than the analytic model's pick, else the analytic pick (a trust region:
  *    smaller predicted gains are within the model's fit error).  No device
  *    work besides the model's forward pass.
+ * The candidates are schedules of the streaming kernel alone.  A pick that is
+ * stored, read from the file or proposed by a cost model is run as it stands: it
+ * also keeps the run off the kernels that the library's rule prefers on small
+ * grids (register tiles, marching passes; see stencil_set_tile), so on grids for
+ * which stencil_run_passes names one of those, a run without a pick is faster
+ * (256^2 radius 1: 0.7 us a step, 12.5 with the best streaming schedule).
  * `chosen` receives the pick; `rows` (capacity `cap`, may be NULL) receives one
  * stencil_timing per candidate and *nrows their number.  With `store` != 0 the
  * pick is kept in the handle and used by later stencil_run calls on the same
@@ -297,7 +305,7 @@ typedef struct {
  * together (not in the paper; a serving-style batch of the paper's sweep).
  * Results equal stencil_run's bit for bit.  The list becomes one CUDA graph that
  * is cached for this exact item list (same pointers, sizes, handles, schedules)
- * and replayed on `stream` by later calls.  Lists with fewer than three grids per
+ * and replayed on `stream` by later calls.  Lists with, on average, fewer than three grids per
  * (dim, radius, dtype, coefficient form) become chains of passes: the 2D grids, on
  * register tiles or streaming passes as in stencil_run, follow one another, and
  * each 3D grid runs on a parallel branch in streaming passes cut for its part of
@@ -340,16 +348,17 @@ int stencil_set_fault_injection(stencil_handle h, int plane, int timeout_ms);
 /* Which kernels run the library's rule.  2D grids run streaming passes or register tiles (128-cell
  * wide tiles held in registers, any number of steps per pass, rows of any length); grids whose rows
  * are not whole 16-byte vectors run the one-step kernel, tiles or, on a padded copy, streaming
- * passes for rows of any length; small 3D grids run one-step passes that march in registers.  All give the same bits, and stencil_run, stencil_run_ex without a
- * schedule and stencil_run_noalloc choose by estimated time; this call is for tests and
- * measurements.  mode 0: choose (the default); -1: the schedule's own kernel only; 1: always where
+ * passes for rows of any length; small 3D grids run one-step passes that march in registers.  All give
+ * the same bits, and stencil_run, stencil_run_ex without a schedule and stencil_run_noalloc choose by
+ * estimated time; this call is for tests and measurements.  mode 0: choose (the default); -1: the schedule's own kernel only; 1: always where
  * they exist, tiles with at most t steps per pass and `rows` rows per thread (0: chosen); 2: never
  * tiles, always padded copies where their kernels exist; 3: 3D marching passes wherever they can.
  * Errors: INVALID_ARG. */
 int stencil_set_tile(stencil_handle h, int mode, int t, int rows);
 
-/* The passes stencil_run would take for this problem when given no schedule (16-byte aligned buffers,
- * memory available): which kernel, how many launches, the steps of the longest one and, for register
+/* The passes stencil_run would take for this problem when given no schedule, where its scratch grids can be
+ * had and buffers are 16-byte aligned (without memory for two padded grids, tiles and marching passes run
+ * on dense rows and padded streaming passes become the one-step kernel): which kernel, how many launches, the steps of the longest one and, for register
  * tiles, the rows per thread.  No device work.  Errors: INVALID_ARG, CUDA. */
 typedef enum {
     STENCIL_PASS_STREAM = 1, /* streaming passes of the schedule */

@@ -217,7 +217,7 @@ def stencil_set_checked(h, on: bool = True) -> int:
 
 def stencil_set_tile(h, mode: int, t: int = 0, rows: int = 0) -> int:
     """Which kernels run the library's rule (see stencil.h): 0 choose, -1 the schedule's own, 1 tiles and
-    padded copies, 2 padded copies."""
+    padded copies, 2 padded copies, 3 marching passes (3D)."""
     return _check(_lib().stencil_set_tile(h, mode, t, rows), "stencil_set_tile")
 
 

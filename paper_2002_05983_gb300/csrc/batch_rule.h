@@ -9,7 +9,7 @@ namespace stn {
 // size does not grow with the steps.
 constexpr int64_t kMaxChainNodes = 20000;
 
-// Lists with fewer than this many grids per kernel class (dimension, radius, storage type, coefficient
+// Lists with, on average, fewer than this many grids per kernel class (dimension, radius, storage type, coefficient
 // form) run as chains.  A persistent class advances all its grids side by side, one tile latency (25-50
 // us) a pass however few they are, and holds its blocks' SMs until it ends; chains take each grid's own
 // fastest passes, but 2D grids one after another, and their graph costs 3-5 us a pass to build.

@@ -1059,7 +1059,7 @@ int run_march(const stencil_plan *h, const void *in, void *out, void *scratch, i
     return 0;
 }
 
-// One step of the one-step kernel (us): 1.9 us and 0.47 us per term and million cells, fitted to
+// One step of the one-step kernel (us): 2.5, and per million cells 1.9 and 0.47 per term, fitted to
 // radius 1 (3D) .. 6 (2D).
 double naive_step_us(const stencil_plan *h, double mcells)
 {
@@ -1412,7 +1412,9 @@ int batch_scratch(const stencil_batch_item *items, int n, const std::vector<int>
     return 0;
 }
 
-// One grid of a batch as a chain of the passes stencil_run would launch.
+// One grid of a batch as a chain of passes: register tiles or streaming passes in 2D, as stencil_run takes
+// them; in 3D streaming passes at every size, because they can be cut for a part of the device, which
+// marching passes are not.
 struct BatchChain {
     int item = 0;
     bool tiles = false;
@@ -1453,8 +1455,9 @@ bool plan_chains(const stencil_batch_item *items, int n, const DevInfo &dev, std
     return stn::batch_as_chains(n, static_cast<int>(classes.size()), nodes);
 }
 
-// One CUDA graph of the grids' chains.  2D passes fill the device, so the 2D grids follow one another
-// on one branch.  A 3D pass of a small grid does not, and cutting it into enough blocks to do so
+// One CUDA graph of the grids' chains.  2D passes of all but small grids fill the device, so the 2D grids
+// follow one another on one branch (lists of many small ones are no chains: batch_rule.h).  A 3D pass of
+// a small grid does not, and cutting it into enough blocks to do so
 // spends most of the planes on halos; every 3D grid has a branch of its own, at high priority, whose
 // passes are cut for 15 times its share of the batch's work, so the 3D chains run beside the 2D
 // one.  Measured on 16 2D + 8 3D grids, 100 steps: 62 ms as persistent launches per kernel class
