@@ -1106,7 +1106,10 @@ bool rag_applicable(const stencil_plan *h, int64_t nx, int64_t ny, int64_t nz, i
     if (h->tile_mode > 0 || h->dim == 2) return true;
     const double mcells = static_cast<double>(nx) * ny * nz * 1e-6;
     const int t = std::max(1, std::min(s.t, iters));
-    const double us = 2.5 + 0.9 * mcells + (iters + t - 1) / t * stream3_pass_us(h->r, t, nx, ny, nz);
+    // the copy and the cell-by-cell stores of the last pass: 1.8 us a million cells (251 x 243 x 237, radius 1: 63 us
+    // for the copy and one pass of 36.5; narrow rows for one or two steps are faster on the one-step kernel: FP16 25
+    // x 651 x 530 53.7 / 56.8 us, shared 18 x 513 x 168 two steps 25.0 / 27.7)
+    const double us = 2.5 + 1.8 * mcells + (iters + t - 1) / t * stream3_pass_us(h->r, t, nx, ny, nz);
     return us < iters * naive_step_us(h, mcells);
 }
 
